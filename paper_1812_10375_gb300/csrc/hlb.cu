@@ -13,6 +13,7 @@
 #include "hlb_march.cuh"
 #include "hlb_split.cuh"
 #include "hlb_energy_walk.cuh"
+#include "hlb_energy_pair.cuh"
 #include "hlb_substep.cuh"
 
 using namespace hlb;
@@ -55,8 +56,8 @@ constexpr int MIN_TILE_Y = 16;  // the shortest variant tile (sizes the partial-
 // threads, and the energy kernel's thread layout (the energy tile is the same).
 struct FlowVariant {
   int ty, nth;
-  int ewalk;   // energy kernel: 0 tile, 1 row walk
-  int ep;      // energy tile: rows per run; walk: segment rows
+  int ewalk;   // energy kernel: 0 tile, 1 row walk, 2 warp-pair walk
+  int ep;      // energy tile: rows per run; walk: segment rows; pair walk: 0, by walk_rows()
   size_t smem;
   const void* single_fn;
   const void* batch_fn;
@@ -66,10 +67,12 @@ struct FlowVariant {
   void (*launch_single)(dim3, size_t, cudaStream_t, const StepArgs&);
   void (*launch_batch)(int, size_t, cudaStream_t, const StepArgs&, const DomArgs*, const int2*, const int*,
                        const float2*);
-  void (*energy_single)(dim3, cudaStream_t, const StepArgs&, int, int);
-  void (*energy_batch)(int, cudaStream_t, const StepArgs&, const DomArgs*, const int2*, const int*, int, int);
-  dim3 egrid(int nx, int ny) const {
-    return ewalk ? dim3((nx + EW_OUT - 1) / EW_OUT, (ny + ep - 1) / ep) : dim3((nx + EN_TX - 1) / EN_TX, (ny + EN_TY - 1) / EN_TY);
+  void (*energy_single)(dim3, cudaStream_t, const StepArgs&, int, int, int);
+  void (*energy_batch)(int, cudaStream_t, const StepArgs&, const DomArgs*, const int2*, const int*, int, int, int);
+  // rows: the pair walk's segment rows
+  dim3 egrid(int nx, int ny, int rows) const {
+    const int L = ewalk == 2 ? rows : (ewalk ? ep : EN_TY);
+    return dim3((nx + EN_TX - 1) / EN_TX, (ny + L - 1) / L);
   }
 };
 template <int TY, int NTH, int MINB, bool RP>
@@ -82,22 +85,29 @@ void launch_flow_batch(int blocks, size_t smem, cudaStream_t s, const StepArgs& 
   k_flow_batch<TY, NTH, MINB, RP><<<blocks, NTH, smem, s>>>(phys, desc, blk, act, lag);
 }
 template <int R, int NPH, int MINB>
-void launch_energy_single(dim3 grid, cudaStream_t s, const StepArgs& a, int sub, int nsub) {
+void launch_energy_single(dim3 grid, cudaStream_t s, const StepArgs& a, int sub, int nsub, int) {
   k_energy<R, NPH, MINB><<<grid, 64 * NPH, energy_smem_bytes(), s>>>(a, sub, nsub);
 }
 template <int R, int NPH, int MINB>
 void launch_energy_batch(int blocks, cudaStream_t s, const StepArgs& phys, const DomArgs* desc, const int2* blk,
-                         const int* act, int sub, int nsub) {
+                         const int* act, int sub, int nsub, int) {
   k_energy_batch<R, NPH, MINB><<<blocks, 64 * NPH, energy_smem_bytes(), s>>>(phys, desc, blk, act, sub, nsub);
 }
 template <int L, int MINB, int PF>
-void launch_walk_single(dim3 grid, cudaStream_t s, const StepArgs& a, int sub, int nsub) {
+void launch_walk_single(dim3 grid, cudaStream_t s, const StepArgs& a, int sub, int nsub, int) {
   k_energy_walk<L, MINB, PF><<<grid, EW_W, 0, s>>>(a, sub, nsub);
 }
 template <int L, int MINB, int PF>
 void launch_walk_batch(int blocks, cudaStream_t s, const StepArgs& phys, const DomArgs* desc, const int2* blk,
-                       const int* act, int sub, int nsub) {
+                       const int* act, int sub, int nsub, int) {
   k_energy_walk_batch<L, MINB, PF><<<blocks, EW_W, 0, s>>>(phys, desc, blk, act, sub, nsub);
+}
+void launch_pair_single(dim3 grid, cudaStream_t s, const StepArgs& a, int sub, int nsub, int rows) {
+  k_energy_pair<<<grid, 32, 0, s>>>(a, rows, sub, nsub);
+}
+void launch_pair_batch(int blocks, cudaStream_t s, const StepArgs& phys, const DomArgs* desc, const int2* blk,
+                       const int* act, int sub, int nsub, int rows) {
+  k_energy_pair_batch<<<blocks, 32, 0, s>>>(phys, desc, blk, act, rows, sub, nsub);
 }
 #define HLB_SPLIT_TILE(TY, NTH, MINB, RP, ER, ENPH, EMINB)                                                      \
   FlowVariant{TY, NTH, 0, ER, flow_smem_bytes<TY>(), (const void*)k_flow<TY, NTH, MINB, RP>,                    \
@@ -111,7 +121,12 @@ void launch_walk_batch(int blocks, cudaStream_t s, const StepArgs& phys, const D
               (const void*)k_energy_walk_batch<L, EMINB, PF>, 0, launch_flow_single<TY, NTH, MINB, RP>,       \
               launch_flow_batch<TY, NTH, MINB, RP>, launch_walk_single<L, EMINB, PF>,                         \
               launch_walk_batch<L, EMINB, PF>},
-const FlowVariant FLOWS[] = {HLB_SPLIT_VARIANTS(HLB_SPLIT_TILE, HLB_SPLIT_WALK)};
+#define HLB_SPLIT_PAIR(TY, NTH, MINB, RP)                                                                       \
+  FlowVariant{TY, NTH, 2, 0, flow_smem_bytes<TY>(), (const void*)k_flow<TY, NTH, MINB, RP>,                     \
+              (const void*)k_flow_batch<TY, NTH, MINB, RP>, (const void*)k_energy_pair,                       \
+              (const void*)k_energy_pair_batch, 0, launch_flow_single<TY, NTH, MINB, RP>,                     \
+              launch_flow_batch<TY, NTH, MINB, RP>, launch_pair_single, launch_pair_batch},
+const FlowVariant FLOWS[] = {HLB_SPLIT_VARIANTS(HLB_SPLIT_TILE, HLB_SPLIT_WALK, HLB_SPLIT_PAIR)};
 constexpr int NSPLIT = (int)(sizeof(FLOWS) / sizeof(FLOWS[0]));
 constexpr int MIN_FLOW_TY = 8;  // the shortest flow tile (sizes the flow partial-sum slots)
 
@@ -143,8 +158,37 @@ dim3 grid_of(int nx, int ny, int W, int top_bc, int v) {
   return dim3((nx + TILE_X - 1) / TILE_X, (ny + VARIANTS[t].ty - 1) / VARIANTS[t].ty);
 }
 // The largest energy grid of any split variant (sizes the energy partial-sum slots).
-dim3 energy_grid_of(int nx, int ny) { return dim3((nx + EN_TX - 1) / EN_TX, (ny + EN_TY - 1) / EN_TY); }
-static_assert(EW_OUT == EN_TX, "walk strips and energy tiles share the column split");
+constexpr int MIN_WALK_ROWS = 4;
+dim3 energy_grid_of(int nx, int ny) {
+  return dim3((nx + EN_TX - 1) / EN_TX, (ny + MIN_WALK_ROWS - 1) / MIN_WALK_ROWS);
+}
+static_assert(EW_OUT == EN_TX && EP_OUT == EN_TX, "walk strips and energy tiles share the column split");
+
+// Segment rows of the one-warp energy walk for n lattices (strips of EP_OUT
+// columns, ny rows each): the smallest height at which every segment is resident at
+// once.  A warp's rows follow one another (0.30 us a row alone, 0.58 us with two
+// warps on a scheduler), so short segments win until the chip is full; beyond that a
+// second wave costs more than taller segments: the 32-domain sweep took 0.0594 ms
+// with 1,142 segments of 86 rows, 0.070 with 901 of 112 and 0.072 with 1,815 of 54;
+// 14 lattices of 400 x 600 0.047 ms with 1,120 of 60, 0.055 with 1,792 of 38.
+constexpr int NUM_SMS = 152;
+int walk_rows(int n, const int* strips, const int* ny) {
+  auto segments = [&](int L) {
+    long long w = 0;
+    for (int i = 0; i < n; ++i) w += (long long)strips[i] * ((ny[i] + L - 1) / L);
+    return w;
+  };
+  constexpr long long SLOTS = (long long)NUM_SMS * EP_CTAS;
+  int lo = MIN_WALK_ROWS, hi = 256;  // more segments than that allows: several waves, 3% halo rows
+  while (lo < hi) {
+    const int mid = lo + (hi - lo) / 2;
+    if (segments(mid) <= SLOTS)
+      hi = mid;
+    else
+      lo = mid + 1;
+  }
+  return lo;
+}
 size_t flow_part_slots(int nx, int ny, int W, int top_bc) {
   return (size_t)((nx + FL_TX - 1) / FL_TX) * ((fluid_rows_of(ny, W, top_bc) + MIN_FLOW_TY - 1) / MIN_FLOW_TY);
 }
@@ -341,6 +385,7 @@ struct hlb_domain {
   double* fpart = nullptr;
   double* epart = nullptr;
   dim3 egrid;
+  int erows = 64;  // segment rows of the pair walk
   int parity = 0;
   long long steps = 0;
   bool fields_set = false;
@@ -359,7 +404,7 @@ namespace {
 void set_variant_grids(hlb_domain* d, int v) {
   d->variant = v;
   d->grid = grid_of(d->p.nx, d->p.ny, d->p.wall_rows, d->p.top_bc, v);
-  d->egrid = is_split(v) ? FLOWS[v].egrid(d->p.nx, d->p.ny) : energy_grid_of(d->p.nx, d->p.ny);
+  d->egrid = is_split(v) ? FLOWS[v].egrid(d->p.nx, d->p.ny, d->erows) : energy_grid_of(d->p.nx, d->p.ny);
 }
 
 }  // namespace
@@ -422,7 +467,7 @@ hlb_status launch_split_step(hlb_domain* d, cudaEvent_t after_flow = nullptr, cu
   fv.launch_single(d->grid, fv.smem, d->stream, a);
   if (after_flow && cudaEventRecord(after_flow, d->stream) != cudaSuccess) return HLB_ECUDA;
   const int nsub = d->p.n_sub;
-  for (int s = 1; s <= nsub; ++s) fv.energy_single(d->egrid, d->stream, a, s, nsub);
+  for (int s = 1; s <= nsub; ++s) fv.energy_single(d->egrid, d->stream, a, s, nsub, d->erows);
   if (after_energy && cudaEventRecord(after_energy, d->stream) != cudaSuccess) return HLB_ECUDA;
   k_reduce_split<<<1, 256, 0, d->stream>>>(d->fpart, (int)(d->grid.x * d->grid.y), d->epart,
                                            (int)(d->egrid.x * d->egrid.y), d->state, 1.0 / (double)d->n_fluid,
@@ -570,6 +615,8 @@ hlb_status init_domain(hlb_domain* d, const hlb_params* p, char* ws, cudaStream_
   }
   const int fluid_rows = q.ny - q.wall_rows - (q.top_bc == HLB_TOP_WALL ? 1 : 0);
   d->n_fluid = (long long)fluid_rows * q.nx;
+  const int strips = (q.nx + EP_OUT - 1) / EP_OUT;
+  d->erows = walk_rows(1, &strips, &q.ny);
   // the split step for the finite-volume scheme; the fused tiled kernel for the isotropic one
   set_variant_grids(d, q.diffusion == HLB_DIFF_FV ? 0 : FIRST_TILED);
   d->smem = smem_bytes();
@@ -848,14 +895,14 @@ hlb_status batch_launch_lanes(hlb_batch* b, const DomArgs* desc) {
   cudaStream_t a = b->stream, s2 = b->side[0];
   fv.launch_batch(b->lane_blk, fv.smem, a, b->phys, desc, b->d_blk, b->d_active, b->d_lag);
   if (cudaEventRecord(b->ev_lane, a) != cudaSuccess) return HLB_ECUDA;
-  for (int s = 1; s <= nsub; ++s) fv.energy_batch(b->lane_eblk, a, b->phys, desc, b->d_eblk, b->d_active, s, nsub);
+  for (int s = 1; s <= nsub; ++s) fv.energy_batch(b->lane_eblk, a, b->phys, desc, b->d_eblk, b->d_active, s, nsub, b->dom[0].erows);
   k_reduce_split_batch<<<m, 256, 0, a>>>(b->d_sra, b->d_active, b->d_lag, HIST_CAP);
   if (cudaStreamWaitEvent(s2, b->ev_lane, 0) != cudaSuccess) return HLB_ECUDA;
   fv.launch_batch(b->total_tiles - b->lane_blk, fv.smem, s2, b->phys, desc, b->d_blk + b->lane_blk, b->d_active,
                   b->d_lag);
   for (int s = 1; s <= nsub; ++s)
     fv.energy_batch(b->total_etiles - b->lane_eblk, s2, b->phys, desc, b->d_eblk + b->lane_eblk, b->d_active, s,
-                    nsub);
+                    nsub, b->dom[0].erows);
   k_reduce_split_batch<<<b->n - m, 256, 0, s2>>>(b->d_sra + m, b->d_active + m, b->d_lag + m, HIST_CAP);
   b->lane_pending = true;
   return cudaGetLastError() == cudaSuccess ? HLB_OK : HLB_ECUDA;
@@ -886,7 +933,7 @@ hlb_status batch_launch(hlb_batch* b, cudaEvent_t before, cudaEvent_t after, cud
     if (mid && cudaEventRecord(mid, b->stream) != cudaSuccess) return HLB_ECUDA;
     const int nsub = b->dom[0].p.n_sub;
     for (int s = 1; s <= nsub; ++s)
-      fv.energy_batch(b->total_etiles, b->stream, b->phys, desc, b->d_eblk, b->d_active, s, nsub);
+      fv.energy_batch(b->total_etiles, b->stream, b->phys, desc, b->d_eblk, b->d_active, s, nsub, b->dom[0].erows);
     if (after && cudaEventRecord(after, b->stream) != cudaSuccess) return HLB_ECUDA;
     k_reduce_split_batch<<<b->n, 256, 0, b->stream>>>(b->d_sra, b->d_active, b->d_lag, HIST_CAP);
     if (cudaGetLastError() != cudaSuccess) return HLB_ECUDA;
@@ -1469,6 +1516,13 @@ hlb_status hlb_batch_init(hlb_batch** out, int n, const hlb_params* p, void* d_w
   b->d_eblk = (int2*)(ws + L.eblk);
   b->d_active = (int*)(ws + L.active);
   b->d_lag = (float2*)(ws + L.lag);
+  std::vector<int> strips(n), nys(n);
+  for (int i = 0; i < n; ++i) {
+    strips[i] = (p[i].nx + EP_OUT - 1) / EP_OUT;
+    nys[i] = p[i].ny;
+  }
+  const int erows = walk_rows(n, strips.data(), nys.data());
+  for (int i = 0; i < n; ++i) b->dom[i].erows = erows;
   const hlb_status st = set_batch_variant(b, 0);
   if (st != HLB_OK) {
     delete b;
@@ -1755,7 +1809,7 @@ int hlb_variant_kind(int v) {
 
 int hlb_variant_energy_rows(int v) {
   if (v < 0 || v >= NV_ALL || !is_split(v)) return -1;
-  return FLOWS[v].ewalk ? FLOWS[v].ep : 0;
+  return FLOWS[v].ewalk == 2 ? 64 : (FLOWS[v].ewalk ? FLOWS[v].ep : 0);
 }
 
 const char* hlb_strerror(hlb_status s) {

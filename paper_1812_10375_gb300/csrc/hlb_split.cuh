@@ -51,9 +51,11 @@ constexpr int FL_FW = FL_TX + 2;   // psi frame: the tile and a one-cell ring
 // WALK(TYF, NTHF, MINBF, RP, L, MINB, PF): the row-walking energy kernel over
 // L-row segments, sized for MINB CTAs per SM, its input rows fetched PF rows
 // ahead by asynchronous copies into shared memory (PF = 0: one row ahead into
-// registers).
-#define HLB_SPLIT_VARIANTS(TILE, WALK) \
-  WALK(24, 256, 4, 1, 64, 10, 6) WALK(16, 256, 4, 1, 64, 10, 6) WALK(16, 256, 3, 0, 64, 10, 6) \
+// registers);
+// PAIR(TYF, NTHF, MINBF, RP): the one-warp energy kernel (hlb_energy_pair.cuh), its
+// segment height chosen by the host from the lattices' sizes.
+#define HLB_SPLIT_VARIANTS(TILE, WALK, PAIR) \
+  PAIR(24, 256, 4, 1) WALK(16, 256, 4, 1, 64, 10, 6) WALK(16, 256, 3, 0, 64, 10, 6) \
   WALK(16, 256, 3, 0, 96, 8, 4) WALK(16, 256, 3, 0, 96, 8, 0) TILE(16, 256, 3, 0, 8, 4, 2)
 
 constexpr int EN_TX = 56, EN_TY = 24, EN_H = 4;
