@@ -20,6 +20,7 @@ using namespace hlb;
 
 namespace {
 
+constexpr int NUM_SMS = 152;
 constexpr int TILE_X = TILE_W;  // 52 output columns in a 64-wide frame
 
 // Compiled variants of the fused step kernel (tile height, threads per CTA).
@@ -52,26 +53,29 @@ constexpr int NVARIANTS = (int)(sizeof(VARIANTS) / sizeof(VARIANTS[0]));
 constexpr int TILE_Y = 28;      // the default variant's tile height (variant 0)
 constexpr int MIN_TILE_Y = 16;  // the shortest variant tile (sizes the partial-sum slots)
 
-// Split-step variants (k_flow* then k_energy*): the flow tile's fluid rows and
-// threads, and the energy kernel's thread layout (the energy tile is the same).
-struct FlowVariant {
+// A compiled flow kernel: its tile's fluid rows and threads.
+struct FlowKernel {
   int ty, nth;
-  int ewalk;   // energy kernel: 0 tile, 1 row walk, 2 warp-pair walk
-  int ep;      // energy tile: rows per run; walk: segment rows; pair walk: 0, by walk_rows()
   size_t smem;
   const void* single_fn;
   const void* batch_fn;
-  const void* esingle_fn;
-  const void* ebatch_fn;
-  size_t esmem;  // dynamic shared memory of the energy kernels
   void (*launch_single)(dim3, size_t, cudaStream_t, const StepArgs&);
   void (*launch_batch)(int, size_t, cudaStream_t, const StepArgs&, const DomArgs*, const int2*, const int*,
                        const float2*);
+};
+struct FlowVariant {
+  int fk;      // flow kernel (index into FLOW_KERNELS), or -1: by flow_kernel_for()
+  int ewalk;   // energy kernel: 0 tile, 1 row walk, 2 one-warp walk
+  int ep;      // energy tile: rows per run; walk: segment rows; one-warp walk: 0, by walk_rows()
+  const void* esingle_fn;
+  const void* ebatch_fn;
+  size_t esmem;  // dynamic shared memory of the energy kernels
   void (*energy_single)(dim3, cudaStream_t, const StepArgs&, int, int, int);
   void (*energy_batch)(int, cudaStream_t, const StepArgs&, const DomArgs*, const int2*, const int*, int, int, int);
-  // rows: the pair walk's segment rows
+  // rows of an energy block; rows: the one-warp walk's
+  int erows(int rows) const { return ewalk == 2 ? rows : (ewalk ? ep : EN_TY); }
   dim3 egrid(int nx, int ny, int rows) const {
-    const int L = ewalk == 2 ? rows : (ewalk ? ep : EN_TY);
+    const int L = erows(rows);
     return dim3((nx + EN_TX - 1) / EN_TX, (ny + L - 1) / L);
   }
 };
@@ -109,26 +113,23 @@ void launch_pair_batch(int blocks, cudaStream_t s, const StepArgs& phys, const D
                        const int* act, int sub, int nsub, int rows) {
   k_energy_pair_batch<<<blocks, 32, 0, s>>>(phys, desc, blk, act, rows, sub, nsub);
 }
-#define HLB_SPLIT_TILE(TY, NTH, MINB, RP, ER, ENPH, EMINB)                                                      \
-  FlowVariant{TY, NTH, 0, ER, flow_smem_bytes<TY>(), (const void*)k_flow<TY, NTH, MINB, RP>,                    \
-              (const void*)k_flow_batch<TY, NTH, MINB, RP>, (const void*)k_energy<ER, ENPH, EMINB>,           \
-              (const void*)k_energy_batch<ER, ENPH, EMINB>, energy_smem_bytes(),                              \
-              launch_flow_single<TY, NTH, MINB, RP>, launch_flow_batch<TY, NTH, MINB, RP>,                    \
-              launch_energy_single<ER, ENPH, EMINB>, launch_energy_batch<ER, ENPH, EMINB>},
-#define HLB_SPLIT_WALK(TY, NTH, MINB, RP, L, EMINB, PF)                                                         \
-  FlowVariant{TY, NTH, 1, L, flow_smem_bytes<TY>(), (const void*)k_flow<TY, NTH, MINB, RP>,                     \
-              (const void*)k_flow_batch<TY, NTH, MINB, RP>, (const void*)k_energy_walk<L, EMINB, PF>,         \
-              (const void*)k_energy_walk_batch<L, EMINB, PF>, 0, launch_flow_single<TY, NTH, MINB, RP>,       \
-              launch_flow_batch<TY, NTH, MINB, RP>, launch_walk_single<L, EMINB, PF>,                         \
-              launch_walk_batch<L, EMINB, PF>},
-#define HLB_SPLIT_PAIR(TY, NTH, MINB, RP)                                                                       \
-  FlowVariant{TY, NTH, 2, 0, flow_smem_bytes<TY>(), (const void*)k_flow<TY, NTH, MINB, RP>,                     \
-              (const void*)k_flow_batch<TY, NTH, MINB, RP>, (const void*)k_energy_pair,                       \
-              (const void*)k_energy_pair_batch, 0, launch_flow_single<TY, NTH, MINB, RP>,                     \
-              launch_flow_batch<TY, NTH, MINB, RP>, launch_pair_single, launch_pair_batch},
+#define HLB_FLOW_ENTRY(TY, NTH, MINB, RP)                                                                        \
+  FlowKernel{TY, NTH, flow_smem_bytes<TY>(), (const void*)k_flow<TY, NTH, MINB, RP>,                             \
+             (const void*)k_flow_batch<TY, NTH, MINB, RP>, launch_flow_single<TY, NTH, MINB, RP>,                \
+             launch_flow_batch<TY, NTH, MINB, RP>},
+const FlowKernel FLOW_KERNELS[] = {HLB_FLOW_KERNELS(HLB_FLOW_ENTRY)};
+#define HLB_SPLIT_TILE(FK, ER, ENPH, EMINB)                                                                      \
+  FlowVariant{FK, 0, ER, (const void*)k_energy<ER, ENPH, EMINB>, (const void*)k_energy_batch<ER, ENPH, EMINB>,   \
+              energy_smem_bytes(), launch_energy_single<ER, ENPH, EMINB>, launch_energy_batch<ER, ENPH, EMINB>},
+#define HLB_SPLIT_WALK(FK, L, EMINB, PF)                                                                         \
+  FlowVariant{FK, 1, L, (const void*)k_energy_walk<L, EMINB, PF>, (const void*)k_energy_walk_batch<L, EMINB, PF>, \
+              0, launch_walk_single<L, EMINB, PF>, launch_walk_batch<L, EMINB, PF>},
+#define HLB_SPLIT_PAIR(FK)                                                                                       \
+  FlowVariant{FK, 2, 0, (const void*)k_energy_pair, (const void*)k_energy_pair_batch, 0, launch_pair_single,     \
+              launch_pair_batch},
 const FlowVariant FLOWS[] = {HLB_SPLIT_VARIANTS(HLB_SPLIT_TILE, HLB_SPLIT_WALK, HLB_SPLIT_PAIR)};
 constexpr int NSPLIT = (int)(sizeof(FLOWS) / sizeof(FLOWS[0]));
-constexpr int MIN_FLOW_TY = 8;  // the shortest flow tile (sizes the flow partial-sum slots)
+constexpr int MIN_FLOW_TY = 4;  // the shortest flow tile (sizes the flow partial-sum slots)
 
 // Variant numbering: [0, NSPLIT) split step, then the fused tiled kernels
 // (VARIANTS), then the row-marching kernels (k_march*: segments of
@@ -147,10 +148,11 @@ size_t march_smem(int nx) { return (size_t)march_smem_floats(nx) * sizeof(float)
 
 int fluid_rows_of(int ny, int W, int top_bc) { return fluid_end(ny, top_bc) - W; }
 
-// Launch grid of the step kernel of variant v (the flow kernel for a split variant).
-dim3 grid_of(int nx, int ny, int W, int top_bc, int v) {
+// Launch grid of the step kernel of variant v (the flow kernel, fk by rule, for a
+// split variant).
+dim3 grid_of(int nx, int ny, int W, int top_bc, int v, int fk = 0) {
   if (is_split(v)) {
-    const int ty = FLOWS[v].ty;
+    const int ty = FLOW_KERNELS[FLOWS[v].fk >= 0 ? FLOWS[v].fk : fk].ty;
     return dim3((nx + FL_TX - 1) / FL_TX, (fluid_rows_of(ny, W, top_bc) + ty - 1) / ty);
   }
   if (is_march(v)) return dim3((ny + march_seg(v) - 1) / march_seg(v), 1);
@@ -171,7 +173,6 @@ static_assert(EW_OUT == EN_TX && EP_OUT == EN_TX, "walk strips and energy tiles 
 // second wave costs more than taller segments: the 32-domain sweep took 0.0594 ms
 // with 1,142 segments of 86 rows, 0.070 with 901 of 112 and 0.072 with 1,815 of 54;
 // 14 lattices of 400 x 600 0.047 ms with 1,120 of 60, 0.055 with 1,792 of 38.
-constexpr int NUM_SMS = 152;
 int walk_rows(int n, const int* strips, const int* ny) {
   auto segments = [&](int L) {
     long long w = 0;
@@ -191,6 +192,22 @@ int walk_rows(int n, const int* strips, const int* ny) {
 }
 size_t flow_part_slots(int nx, int ny, int W, int top_bc) {
   return (size_t)((nx + FL_TX - 1) / FL_TX) * ((fluid_rows_of(ny, W, top_bc) + MIN_FLOW_TY - 1) / MIN_FLOW_TY);
+}
+// Flow kernel for n lattices (tiles to a row of tiles, fluid rows): the shortest tile
+// whose CTAs are all resident at once (four per SM), else the 24-row one.  A thread
+// runs through its rows one after the other, so on a chip that is not full short
+// tiles are faster; a full one wants tall tiles, whose psi ring costs less per
+// cell.  Whole steps with tiles of 24, 16, 8 and 4 rows: 64 x 200 25.4, 23.0, 20.6,
+// 19.7 us; 400 x 400 29.3, 27.9, 27.4, 28.1; 48 lattices of 64 to 96 columns 44.7,
+// 41.5, 41.9, 44.1; 14 of 400 x 600 121, 121, 133, 165.
+int flow_kernel_for(int n, const int* tx, const int* rows) {
+  int best = 0;
+  for (int k = 0; k < NFLOW_RULE; ++k) {
+    long long w = 0;
+    for (int i = 0; i < n; ++i) w += (long long)tx[i] * ((rows[i] + FLOW_KERNELS[k].ty - 1) / FLOW_KERNELS[k].ty);
+    if (w <= 4LL * NUM_SMS) best = k;
+  }
+  return best;
 }
 constexpr int GRAPH_STEPS = 16;     // steps per captured graph (even: buffers return to parity 0)
 constexpr int HIST_CAP = 1 << 16;   // wall-flux history entries kept per domain
@@ -385,7 +402,8 @@ struct hlb_domain {
   double* fpart = nullptr;
   double* epart = nullptr;
   dim3 egrid;
-  int erows = 64;  // segment rows of the pair walk
+  int erows = 64;  // segment rows of the one-warp energy walk
+  int fk = 0;      // flow kernel by rule
   int parity = 0;
   long long steps = 0;
   bool fields_set = false;
@@ -400,10 +418,15 @@ struct hlb_domain {
 
 namespace {
 
+const FlowKernel& flow_kernel_of(const hlb_domain* d) {
+  const int fk = is_split(d->variant) ? FLOWS[d->variant].fk : -1;
+  return FLOW_KERNELS[fk >= 0 ? fk : d->fk];
+}
+
 // Variant v for domain d: launch grids of its step kernel(s).
 void set_variant_grids(hlb_domain* d, int v) {
   d->variant = v;
-  d->grid = grid_of(d->p.nx, d->p.ny, d->p.wall_rows, d->p.top_bc, v);
+  d->grid = grid_of(d->p.nx, d->p.ny, d->p.wall_rows, d->p.top_bc, v, d->fk);
   d->egrid = is_split(v) ? FLOWS[v].egrid(d->p.nx, d->p.ny, d->erows) : energy_grid_of(d->p.nx, d->p.ny);
 }
 
@@ -460,18 +483,38 @@ StepArgs args_for(hlb_domain* d, int par) {
   return a;
 }
 
+// The reduction's view of domain d under its split variant.
+SplitReduceArgs reduce_args_of(const hlb_domain* d) {
+  const FlowVariant& fv = FLOWS[is_split(d->variant) ? d->variant : 0];
+  const int ty = flow_kernel_of(d).ty, rows = fv.erows(d->erows);
+  SplitReduceArgs r;
+  r.fpart = d->fpart;
+  r.epart = d->epart;
+  r.state = d->state;
+  r.hist = d->hist;
+  r.nf = (int)(d->grid.x * d->grid.y);
+  r.ne = (int)(d->egrid.x * d->egrid.y);
+  r.tx = (int)d->grid.x;
+  r.strips = (int)d->egrid.x;
+  r.ut0 = (d->p.ny - 2 - d->p.wall_rows) / ty * r.tx;
+  r.qi0 = d->p.wall_rows / rows * r.strips;
+  r.qt0 = d->p.top_bc == HLB_TOP_WALL ? (d->p.ny - 2) / rows * r.strips : -1;
+  r.inv_nfluid = 1.0 / (double)d->n_fluid;
+  r.inv_nx = 1.0 / (double)d->p.nx;
+  return r;
+}
+
 // One step of the split form: the flow kernel, N energy sub-steps, the reduction.
 hlb_status launch_split_step(hlb_domain* d, cudaEvent_t after_flow = nullptr, cudaEvent_t after_energy = nullptr) {
   const StepArgs a = args_for(d, d->parity);
   const FlowVariant& fv = FLOWS[d->variant];
-  fv.launch_single(d->grid, fv.smem, d->stream, a);
+  const FlowKernel& fl = flow_kernel_of(d);
+  fl.launch_single(d->grid, fl.smem, d->stream, a);
   if (after_flow && cudaEventRecord(after_flow, d->stream) != cudaSuccess) return HLB_ECUDA;
   const int nsub = d->p.n_sub;
   for (int s = 1; s <= nsub; ++s) fv.energy_single(d->egrid, d->stream, a, s, nsub, d->erows);
   if (after_energy && cudaEventRecord(after_energy, d->stream) != cudaSuccess) return HLB_ECUDA;
-  k_reduce_split<<<1, 256, 0, d->stream>>>(d->fpart, (int)(d->grid.x * d->grid.y), d->epart,
-                                           (int)(d->egrid.x * d->egrid.y), d->state, 1.0 / (double)d->n_fluid,
-                                           1.0 / (double)d->p.nx, d->hist, HIST_CAP);
+  k_reduce_split<<<1, 256, 0, d->stream>>>(reduce_args_of(d), HIST_CAP);
   if (cudaGetLastError() != cudaSuccess) return HLB_ECUDA;
   d->parity ^= 1;
   d->steps += 1;
@@ -615,8 +658,9 @@ hlb_status init_domain(hlb_domain* d, const hlb_params* p, char* ws, cudaStream_
   }
   const int fluid_rows = q.ny - q.wall_rows - (q.top_bc == HLB_TOP_WALL ? 1 : 0);
   d->n_fluid = (long long)fluid_rows * q.nx;
-  const int strips = (q.nx + EP_OUT - 1) / EP_OUT;
+  const int strips = (q.nx + EP_OUT - 1) / EP_OUT, tx = (q.nx + FL_TX - 1) / FL_TX;
   d->erows = walk_rows(1, &strips, &q.ny);
+  d->fk = flow_kernel_for(1, &tx, &fluid_rows);
   // the split step for the finite-volume scheme; the fused tiled kernel for the isotropic one
   set_variant_grids(d, q.diffusion == HLB_DIFF_FV ? 0 : FIRST_TILED);
   d->smem = smem_bytes();
@@ -673,11 +717,9 @@ hlb_status init_domain(hlb_domain* d, const hlb_params* p, char* ws, cudaStream_
   a.fpart = d->fpart;
   a.epart = d->epart;
 
-  for (int v = 0; v < NSPLIT; ++v) {
-    if (cudaFuncSetAttribute(FLOWS[v].single_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FLOWS[v].smem) !=
-            cudaSuccess ||
-        cudaFuncSetAttribute(FLOWS[v].batch_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FLOWS[v].smem) !=
-            cudaSuccess)
+  for (const FlowKernel& k : FLOW_KERNELS) {
+    if (cudaFuncSetAttribute(k.single_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem) != cudaSuccess ||
+        cudaFuncSetAttribute(k.batch_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem) != cudaSuccess)
       return HLB_ECUDA;
   }
   for (int v = 0; v < NSPLIT; ++v) {
@@ -847,14 +889,7 @@ hlb_status upload_tables(hlb_batch* b) {
     ra[i].nblk = (int)(d->grid.x * d->grid.y);
     ra[i].inv_nfluid = 1.0 / (double)d->n_fluid;
     ra[i].inv_nx = 1.0 / (double)d->p.nx;
-    sra[i].fpart = d->fpart;
-    sra[i].epart = d->epart;
-    sra[i].state = d->state;
-    sra[i].hist = d->hist;
-    sra[i].nf = (int)(d->grid.x * d->grid.y);
-    sra[i].ne = (int)(d->egrid.x * d->egrid.y);
-    sra[i].inv_nfluid = ra[i].inv_nfluid;
-    sra[i].inv_nx = ra[i].inv_nx;
+    sra[i] = reduce_args_of(d);
   }
   if (cudaMemcpyAsync(b->d_desc, desc.data(), desc.size() * sizeof(DomArgs), cudaMemcpyHostToDevice, b->stream) !=
           cudaSuccess ||
@@ -893,12 +928,13 @@ hlb_status batch_launch_lanes(hlb_batch* b, const DomArgs* desc) {
   const int nsub = b->dom[0].p.n_sub;
   const int m = b->lane_split;
   cudaStream_t a = b->stream, s2 = b->side[0];
-  fv.launch_batch(b->lane_blk, fv.smem, a, b->phys, desc, b->d_blk, b->d_active, b->d_lag);
+  const FlowKernel& fl = flow_kernel_of(&b->dom[0]);
+  fl.launch_batch(b->lane_blk, fl.smem, a, b->phys, desc, b->d_blk, b->d_active, b->d_lag);
   if (cudaEventRecord(b->ev_lane, a) != cudaSuccess) return HLB_ECUDA;
   for (int s = 1; s <= nsub; ++s) fv.energy_batch(b->lane_eblk, a, b->phys, desc, b->d_eblk, b->d_active, s, nsub, b->dom[0].erows);
   k_reduce_split_batch<<<m, 256, 0, a>>>(b->d_sra, b->d_active, b->d_lag, HIST_CAP);
   if (cudaStreamWaitEvent(s2, b->ev_lane, 0) != cudaSuccess) return HLB_ECUDA;
-  fv.launch_batch(b->total_tiles - b->lane_blk, fv.smem, s2, b->phys, desc, b->d_blk + b->lane_blk, b->d_active,
+  fl.launch_batch(b->total_tiles - b->lane_blk, fl.smem, s2, b->phys, desc, b->d_blk + b->lane_blk, b->d_active,
                   b->d_lag);
   for (int s = 1; s <= nsub; ++s)
     fv.energy_batch(b->total_etiles - b->lane_eblk, s2, b->phys, desc, b->d_eblk + b->lane_eblk, b->d_active, s,
@@ -929,7 +965,8 @@ hlb_status batch_launch(hlb_batch* b, cudaEvent_t before, cudaEvent_t after, cud
   }
   if (is_split(b->variant)) {
     const FlowVariant& fv = FLOWS[b->variant];
-    fv.launch_batch(b->total_tiles, fv.smem, b->stream, b->phys, desc, b->d_blk, b->d_active, b->d_lag);
+    const FlowKernel& fl = flow_kernel_of(&b->dom[0]);
+    fl.launch_batch(b->total_tiles, fl.smem, b->stream, b->phys, desc, b->d_blk, b->d_active, b->d_lag);
     if (mid && cudaEventRecord(mid, b->stream) != cudaSuccess) return HLB_ECUDA;
     const int nsub = b->dom[0].p.n_sub;
     for (int s = 1; s <= nsub; ++s)
@@ -1120,7 +1157,7 @@ hlb_status set_batch_variant(hlb_batch* b, int v) {
     for (int i = 0; i < b->n; ++i)
       for (int t = b->tile_off[i]; t < b->tile_off[i + 1]; ++t) b->blk.push_back(make_int2(i, t - b->tile_off[i]));
   }
-  b->smem = is_split(v) ? FLOWS[v].smem : (is_march(v) ? march_smem(MARCH_MAX_NX) : VARIANTS[tiled_index(v)].smem);
+  b->smem = is_split(v) ? flow_kernel_of(&b->dom[0]).smem : (is_march(v) ? march_smem(MARCH_MAX_NX) : VARIANTS[tiled_index(v)].smem);
   const hlb_status st = lane_setup(b);
   if (st != HLB_OK) return st;
   batch_drop_graph(b);
@@ -1516,13 +1553,18 @@ hlb_status hlb_batch_init(hlb_batch** out, int n, const hlb_params* p, void* d_w
   b->d_eblk = (int2*)(ws + L.eblk);
   b->d_active = (int*)(ws + L.active);
   b->d_lag = (float2*)(ws + L.lag);
-  std::vector<int> strips(n), nys(n);
+  std::vector<int> strips(n), nys(n), tx(n), rows(n);
   for (int i = 0; i < n; ++i) {
     strips[i] = (p[i].nx + EP_OUT - 1) / EP_OUT;
     nys[i] = p[i].ny;
+    tx[i] = (p[i].nx + FL_TX - 1) / FL_TX;
+    rows[i] = fluid_rows_of(p[i].ny, p[i].wall_rows, p[i].top_bc);
   }
-  const int erows = walk_rows(n, strips.data(), nys.data());
-  for (int i = 0; i < n; ++i) b->dom[i].erows = erows;
+  const int erows = walk_rows(n, strips.data(), nys.data()), fk = flow_kernel_for(n, tx.data(), rows.data());
+  for (int i = 0; i < n; ++i) {
+    b->dom[i].erows = erows;
+    b->dom[i].fk = fk;
+  }
   const hlb_status st = set_batch_variant(b, 0);
   if (st != HLB_OK) {
     delete b;
@@ -1787,8 +1829,9 @@ int hlb_tile_variants(int* h_tile_w, int* h_tile_h, int* h_threads, int max_out)
     // thread per column (0)
     if (is_split(v)) {
       if (h_tile_w) h_tile_w[v] = FL_TX;
-      if (h_tile_h) h_tile_h[v] = FLOWS[v].ty;
-      if (h_threads) h_threads[v] = FLOWS[v].nth;
+      const FlowKernel& k = FLOW_KERNELS[FLOWS[v].fk >= 0 ? FLOWS[v].fk : 0];
+      if (h_tile_h) h_tile_h[v] = k.ty;
+      if (h_threads) h_threads[v] = k.nth;
     } else if (is_march(v)) {
       if (h_tile_w) h_tile_w[v] = 0;
       if (h_tile_h) h_tile_h[v] = march_seg(v);

@@ -42,21 +42,22 @@ enum { EP_QB = 0, EP_QT, EP_QI, EP_E, NEPART };
 
 constexpr int FL_TX = 64;          // flow tile width
 constexpr int FL_FW = FL_TX + 2;   // psi frame: the tile and a one-cell ring
-// Compiled split-step variants: flow tile (fluid rows, threads per CTA, CTAs
-// per SM) and energy layout (rows per thread run, runs, CTAs per SM).
-// TYF, NTHF, MINBF: the flow tile's fluid rows, threads and CTAs per SM; RP:
-// the flow kernel pulls its own cells again after the barrier instead of
-// holding their populations in registers (fewer registers, more CTAs per SM).
-// TILE(TYF, NTHF, MINBF, RP, R, NPH, MINB): the energy tile of R-row runs;
-// WALK(TYF, NTHF, MINBF, RP, L, MINB, PF): the row-walking energy kernel over
-// L-row segments, sized for MINB CTAs per SM, its input rows fetched PF rows
-// ahead by asynchronous copies into shared memory (PF = 0: one row ahead into
-// registers);
-// PAIR(TYF, NTHF, MINBF, RP): the one-warp energy kernel (hlb_energy_pair.cuh), its
-// segment height chosen by the host from the lattices' sizes.
+// Compiled flow kernels: X(TYF, NTHF, MINBF, RP): the flow tile's fluid rows, threads
+// and CTAs per SM; RP: the kernel pulls its own cells again after the barrier
+// instead of holding their populations in registers (fewer registers, more CTAs
+// per SM).  The first NFLOW_RULE are chosen from by the lattices' sizes.
+#define HLB_FLOW_KERNELS(X) \
+  X(24, 256, 4, 1) X(16, 256, 4, 1) X(8, 256, 4, 1) X(4, 256, 4, 1) X(16, 256, 3, 0)
+constexpr int NFLOW_RULE = 4;
+// Compiled split-step variants: flow kernel (index above, -1: by size) and
+// TILE(FK, R, NPH, MINB): the energy tile of R-row runs;
+// WALK(FK, L, MINB, PF): the two-warp row-walking energy kernel over L-row segments,
+// sized for MINB CTAs per SM, its input rows fetched PF rows ahead by
+// asynchronous copies into shared memory (PF = 0: one row ahead into registers);
+// PAIR(FK): the one-warp energy kernel (hlb_energy_pair.cuh), its segment height
+// chosen by the host from the lattices' sizes.
 #define HLB_SPLIT_VARIANTS(TILE, WALK, PAIR) \
-  PAIR(24, 256, 4, 1) WALK(16, 256, 4, 1, 64, 10, 6) WALK(16, 256, 3, 0, 64, 10, 6) \
-  WALK(16, 256, 3, 0, 96, 8, 4) WALK(16, 256, 3, 0, 96, 8, 0) TILE(16, 256, 3, 0, 8, 4, 2)
+  PAIR(-1) WALK(1, 64, 10, 6) WALK(4, 64, 10, 6) WALK(4, 96, 8, 4) WALK(4, 96, 8, 0) TILE(4, 8, 4, 2)
 
 constexpr int EN_TX = 56, EN_TY = 24, EN_H = 4;
 constexpr int EN_FW = EN_TX + 2 * EN_H;  // 64 frame columns, one per thread
@@ -802,82 +803,103 @@ __global__ void __launch_bounds__(64 * NPH, MINB) k_energy_batch(const StepArgs 
 }
 
 // ------------------------------------------------------------- reduction
-// Sums the flow and energy tiles' partials of one domain (one CTA) and updates
-// the record: lagged mean density (Eq. 9) and outlet velocity for the next
-// step, diagnostics, running sums, flux history.
-__device__ __forceinline__ void reduce_split_block(const double* __restrict__ fpart, int nf,
-                                                   const double* __restrict__ epart, int ne, DevState* st,
-                                                   double inv_nfluid, double inv_nx, double* hist, int hist_cap,
-                                                   float2* lag) {
-  __shared__ double s_red[8][NFPART + NEPART];
-  double v[NFPART + NEPART];
-#pragma unroll
-  for (int q = 0; q < NFPART + NEPART; ++q) v[q] = 0.0;
-  for (int b = threadIdx.x; b < nf; b += blockDim.x) {
-#pragma unroll
-    for (int q = 0; q < NFPART; ++q) v[q] += fpart[(long long)b * NFPART + q];
-  }
-  for (int b = threadIdx.x; b < ne; b += blockDim.x) {
-#pragma unroll
-    for (int q = 0; q < NEPART; ++q) v[NFPART + q] += epart[(long long)b * NEPART + q];
-  }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int q = 0; q < NFPART + NEPART; ++q) {
-    const double s = warp_sum(v[q]);
-    if (lane == 0) s_red[warp][q] = s;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double s[NFPART + NEPART];
-#pragma unroll
-    for (int q = 0; q < NFPART + NEPART; ++q) {
-      s[q] = 0.0;
-      for (int w = 0; w < 8; ++w) s[q] += s_red[w][q];
-    }
-    st->rho_ave_prev = st->rho_ave;
-    st->rho_ave = s[FP_MASS] * inv_nfluid;
-    const double ut = s[FP_UTOP] * inv_nx;
-    st->u_top = ut;
-    st->U = ut > 0.0 ? ut : 0.0;
-    st->Uc = st->U / (1.0 + st->U);
-    st->step += 1;
-    st->mass = s[FP_MASS];
-    st->energy = s[NFPART + EP_E];
-    st->q_bottom = s[NFPART + EP_QB] * inv_nx;
-    st->q_top = s[NFPART + EP_QT] * inv_nx;
-    st->q_interface = s[NFPART + EP_QI] * inv_nx;
-    st->q_sum += st->q_bottom;
-    st->q_count += 1;
-    st->vcov = s[FP_VCOV] * inv_nx;
-    st->vcov_sum += st->vcov;
-    if (hist && st->hist_len < hist_cap) hist[st->hist_len++] = st->q_bottom;
-    if (lag) *lag = make_float2((float)st->Uc, (float)st->rho_ave);
-  }
-}
-
-__global__ void __launch_bounds__(256) k_reduce_split(const double* __restrict__ fpart, int nf,
-                                                       const double* __restrict__ epart, int ne, DevState* st,
-                                                       double inv_nfluid, double inv_nx, double* hist, int hist_cap) {
-  reduce_split_block(fpart, nf, epart, ne, st, inv_nfluid, inv_nx, hist, hist_cap, nullptr);
-}
-
+// Where a domain's partial sums lie: the flow tiles' (nf, tx tiles to a row of
+// tiles) and the energy blocks' (ne, strips to a row of blocks).  Every block has
+// mass or energy; the other quantities come from one row of blocks each: the
+// vapour count of row W from the first row of flow tiles, u_y of row ny - 2 from
+// the tiles at ut0, q_bottom from the first row of energy blocks, q_interface and
+// q_top from the blocks at qi0 and qt0.
 struct SplitReduceArgs {
   const double* fpart;
   const double* epart;
   DevState* state;
   double* hist;
-  int nf, ne;
+  int nf, ne, tx, strips, ut0, qi0, qt0;
   double inv_nfluid, inv_nx;
 };
+
+// Sums the flow and energy kernels' partials of one domain (one CTA) and updates
+// the record: lagged mean density (Eq. 9) and outlet velocity for the next
+// step, diagnostics, running sums, flux history.  The FP64 pipe (a warp's add takes
+// 16 cycles of an SM's) and the record's load latency bound it: mass and energy are
+// added in four-entry strides and folded by one warp each, the one-row quantities
+// by a warp each, and the record's old values are fetched before the sums.
+// One CTA adding seven sums of every partial took 8.5 us of a 33 us step of one
+// 400 x 400 lattice (912 partials); so ordered, 5.
+__device__ __forceinline__ void reduce_split_block(const SplitReduceArgs& r, int hist_cap, float2* lag) {
+  enum { R_MASS, R_ENERGY, R_VCOV, R_UTOP, R_QB, R_QT, R_QI, NR };
+  __shared__ double s_part[2][256];
+  __shared__ double s_sum[NR];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  DevState* const st = r.state;
+  DevState old;
+  if (tid == 0) old = *st;
+  double m = 0.0, e = 0.0;
+  for (int b = tid; b < r.nf; b += 256) m += r.fpart[(long long)b * NFPART + FP_MASS];
+  for (int b = tid; b < r.ne; b += 256) e += r.epart[(long long)b * NEPART + EP_E];
+  s_part[0][tid] = m;
+  s_part[1][tid] = e;
+  if (warp >= R_VCOV && warp < NR) {
+    const bool flow = warp <= R_UTOP;
+    const int n = flow ? r.tx : r.strips;
+    const int at = warp == R_UTOP ? r.ut0 : (warp == R_QT ? r.qt0 : (warp == R_QI ? r.qi0 : 0));
+    const int q = warp == R_VCOV ? FP_VCOV : (warp == R_UTOP ? FP_UTOP : (warp == R_QB ? EP_QB : (warp == R_QT ? EP_QT : EP_QI)));
+    const double* p = flow ? r.fpart : r.epart;
+    const int stride = flow ? NFPART : NEPART;
+    double v = 0.0;
+    if (at >= 0)
+      for (int b = lane; b < n; b += 32) v += p[(long long)(at + b) * stride + q];
+    v = warp_sum(v);
+    if (lane == 0) s_sum[warp] = v;
+  }
+  __syncthreads();
+  if (warp < 2) {
+    double v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = s_part[warp][lane + 32 * k];
+    const double t = warp_sum(((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7])));
+    if (lane == 0) s_sum[warp] = t;
+  }
+  __syncthreads();
+  if (tid == 0) {
+    const double rho_ave = s_sum[R_MASS] * r.inv_nfluid;
+    const double ut = s_sum[R_UTOP] * r.inv_nx;
+    const double U = ut > 0.0 ? ut : 0.0;
+    const double Uc = U > 0.0 ? U / (1.0 + U) : 0.0;
+    if (lag) *lag = make_float2((float)Uc, (float)rho_ave);
+    const double qb = s_sum[R_QB] * r.inv_nx, vcov = s_sum[R_VCOV] * r.inv_nx;
+    st->rho_ave_prev = old.rho_ave;
+    st->rho_ave = rho_ave;
+    st->u_top = ut;
+    st->U = U;
+    st->Uc = Uc;
+    st->step = old.step + 1;
+    st->mass = s_sum[R_MASS];
+    st->energy = s_sum[R_ENERGY];
+    st->q_bottom = qb;
+    st->q_top = s_sum[R_QT] * r.inv_nx;
+    st->q_interface = s_sum[R_QI] * r.inv_nx;
+    st->q_sum = old.q_sum + qb;
+    st->q_count = old.q_count + 1;
+    st->vcov = vcov;
+    st->vcov_sum = old.vcov_sum + vcov;
+    if (r.hist && old.hist_len < hist_cap) {
+      r.hist[old.hist_len] = qb;
+      st->hist_len = old.hist_len + 1;
+    }
+  }
+}
+
+__global__ void __launch_bounds__(256) k_reduce_split(const __grid_constant__ SplitReduceArgs r, int hist_cap) {
+  reduce_split_block(r, hist_cap, nullptr);
+}
 
 __global__ void __launch_bounds__(256) k_reduce_split_batch(const SplitReduceArgs* __restrict__ ra,
                                                              const int* __restrict__ active, float2* lag,
                                                              int hist_cap) {
   const int d = blockIdx.x;
   if (!active[d]) return;
-  const SplitReduceArgs r = ra[d];
-  reduce_split_block(r.fpart, r.nf, r.epart, r.ne, r.state, r.inv_nfluid, r.inv_nx, r.hist, hist_cap, lag + d);
+  reduce_split_block(ra[d], hist_cap, lag + d);
 }
 
 }  // namespace hlb
