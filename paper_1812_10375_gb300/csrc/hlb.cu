@@ -106,12 +106,24 @@ void launch_walk_batch(int blocks, cudaStream_t s, const StepArgs& phys, const D
                        const int* act, int sub, int nsub, int) {
   k_energy_walk_batch<L, MINB, PF><<<blocks, EW_W, 0, s>>>(phys, desc, blk, act, sub, nsub);
 }
+// Segments of up to 12 rows run the one-row loop: a warp passes through each line of
+// code a few times only, so that fetching instructions, not issuing them, takes the
+// time.  Whole steps, three-row against one-row loop: 64 x 200 (4 rows) 19.6 and
+// 17.7 us, 385 x 301 with N = 3 (4 rows) 62.7 and 44.3, 48 small lattices (8 rows)
+// 41.6 and 34.0; 400 x 400 with 12 rows 28.6 and 27.6, with 16 rows 29.5 and 30.1.
+bool pair_short(int rows) { return rows <= 12; }
 void launch_pair_single(dim3 grid, cudaStream_t s, const StepArgs& a, int sub, int nsub, int rows) {
-  k_energy_pair<<<grid, 32, 0, s>>>(a, rows, sub, nsub);
+  if (pair_short(rows))
+    k_energy_pair<1><<<grid, 32, 0, s>>>(a, rows, sub, nsub);
+  else
+    k_energy_pair<EP_U><<<grid, 32, 0, s>>>(a, rows, sub, nsub);
 }
 void launch_pair_batch(int blocks, cudaStream_t s, const StepArgs& phys, const DomArgs* desc, const int2* blk,
                        const int* act, int sub, int nsub, int rows) {
-  k_energy_pair_batch<<<blocks, 32, 0, s>>>(phys, desc, blk, act, rows, sub, nsub);
+  if (pair_short(rows))
+    k_energy_pair_batch<1><<<blocks, 32, 0, s>>>(phys, desc, blk, act, rows, sub, nsub);
+  else
+    k_energy_pair_batch<EP_U><<<blocks, 32, 0, s>>>(phys, desc, blk, act, rows, sub, nsub);
 }
 #define HLB_FLOW_ENTRY(TY, NTH, MINB, RP)                                                                        \
   FlowKernel{TY, NTH, flow_smem_bytes<TY>(), (const void*)k_flow<TY, NTH, MINB, RP>,                             \
@@ -125,7 +137,7 @@ const FlowKernel FLOW_KERNELS[] = {HLB_FLOW_KERNELS(HLB_FLOW_ENTRY)};
   FlowVariant{FK, 1, L, (const void*)k_energy_walk<L, EMINB, PF>, (const void*)k_energy_walk_batch<L, EMINB, PF>, \
               0, launch_walk_single<L, EMINB, PF>, launch_walk_batch<L, EMINB, PF>},
 #define HLB_SPLIT_PAIR(FK)                                                                                       \
-  FlowVariant{FK, 2, 0, (const void*)k_energy_pair, (const void*)k_energy_pair_batch, 0, launch_pair_single,     \
+  FlowVariant{FK, 2, 0, (const void*)k_energy_pair<EP_U>, (const void*)k_energy_pair_batch<EP_U>, 0, launch_pair_single,     \
               launch_pair_batch},
 const FlowVariant FLOWS[] = {HLB_SPLIT_VARIANTS(HLB_SPLIT_TILE, HLB_SPLIT_WALK, HLB_SPLIT_PAIR)};
 constexpr int NSPLIT = (int)(sizeof(FLOWS) / sizeof(FLOWS[0]));
@@ -158,6 +170,15 @@ dim3 grid_of(int nx, int ny, int W, int top_bc, int v, int fk = 0) {
   if (is_march(v)) return dim3((ny + march_seg(v) - 1) / march_seg(v), 1);
   const int t = tiled_index(v);
   return dim3((nx + TILE_X - 1) / TILE_X, (ny + VARIANTS[t].ty - 1) / VARIANTS[t].ty);
+}
+// Tile variant of the isotropic scheme: 20-row tiles while they are all resident (two
+// per SM; 120 x 200: 21.3 us a step against 24.7 with 28 rows, 300 x 300 22.2 against
+// 25.8), 28-row ones beyond, whose halo costs less per cell (800 x 400: 35.0 against
+// 39.3 us).
+int fused_tile_for(int nx, int ny) {
+  constexpr int SHORT = 2;
+  const long long n = (long long)((nx + TILE_X - 1) / TILE_X) * ((ny + VARIANTS[SHORT].ty - 1) / VARIANTS[SHORT].ty);
+  return n <= 2 * NUM_SMS ? SHORT : 0;
 }
 // The largest energy grid of any split variant (sizes the energy partial-sum slots).
 constexpr int MIN_WALK_ROWS = 4;
@@ -662,7 +683,7 @@ hlb_status init_domain(hlb_domain* d, const hlb_params* p, char* ws, cudaStream_
   d->erows = walk_rows(1, &strips, &q.ny);
   d->fk = flow_kernel_for(1, &tx, &fluid_rows);
   // the split step for the finite-volume scheme; the fused tiled kernel for the isotropic one
-  set_variant_grids(d, q.diffusion == HLB_DIFF_FV ? 0 : FIRST_TILED);
+  set_variant_grids(d, q.diffusion == HLB_DIFF_FV ? 0 : FIRST_TILED + fused_tile_for(q.nx, q.ny));
   d->smem = smem_bytes();
 
   StepArgs& a = d->base;

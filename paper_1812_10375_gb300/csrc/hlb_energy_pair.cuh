@@ -36,9 +36,9 @@ namespace hlb {
 constexpr int EPW = 64;      // frame columns of a warp
 constexpr int EP_OUT = 56;   // output columns of a strip
 constexpr int EP_H = 4;      // x halo
-constexpr int EP_U = 3;      // rows per pass of the walk's loop
-constexpr int EP_TS = 16;    // slots of the rings of input rows (rows t - 4 .. t + 3 EP_U - 1)
-constexpr int EP_PF = 2;     // groups of EP_U rows fetched ahead
+constexpr int EP_U = 3;      // rows per pass of the throughput form's loop
+constexpr int EP_TS = 16;    // slots of the rings of input rows (rows t - 4 .. t + 8)
+constexpr int EP_PF = 6;     // rows fetched ahead
 constexpr int EP_CTAS = 8;   // resident one-warp CTAs per SM (two per scheduler, at most 255 registers)
 
 struct PairShared {
@@ -86,12 +86,12 @@ struct PairCtx {
   bool own0, own1, last;
 };
 
-// Start the copies of rows t .. t + EP_U - 1 (rows above the lattice repeat row
+// Start the copies of rows t .. t + U - 1 (rows above the lattice repeat row
 // ny - 1; rows below it are not read) into their slots, as one group.
-template <bool VEC>
+template <int U, bool VEC>
 __device__ __forceinline__ void pair_fetch(const StepArgs& A, const PairCtx& C, PairShared& sm, int t) {
 #pragma unroll
-  for (int k = 0; k < EP_U; ++k) {
+  for (int k = 0; k < U; ++k) {
     const int row = t + k;
     if (row < 0) continue;
     const int o = min(row, A.ny - 1) * A.nx, st = row & (EP_TS - 1);
@@ -348,22 +348,44 @@ __device__ __forceinline__ void pair_step(const StepArgs& A, const PairCtx& C, P
   }
 }
 
-// Whether steps t .. t + EP_U - 1 need the boundary rows' tests.
+// Whether steps t .. t + U - 1 need the boundary rows' tests.
+template <int U>
 __device__ __forceinline__ bool pair_bnd(const StepArgs& A, int t) {
-  const int e = t + EP_U - 1;
+  const int e = t + U - 1;
   return t <= 5 || (e >= A.W + 1 && t <= A.W + 4) || e > (A.top_bc == TOP_WALL ? A.ny - 2 : A.ny);
 }
 
-// EP_U steps from row t on
-template <bool BND, bool VEC, bool BATCH>
+// U steps from row t on; U = 1 turns the rings by a row afterwards.
+template <int U, bool BND, bool VEC, bool BATCH>
 __device__ __forceinline__ void pair_group(const StepArgs& A, const PairCtx& C, PairState& S, PairShared& sm, int t) {
   pair_step<0, BND, VEC, BATCH>(A, C, S, sm, t);
-  pair_step<1, BND, VEC, BATCH>(A, C, S, sm, t + 1);
-  pair_step<2, BND, VEC, BATCH>(A, C, S, sm, t + 2);
+  if constexpr (U == 3) {
+    pair_step<1, BND, VEC, BATCH>(A, C, S, sm, t + 1);
+    pair_step<2, BND, VEC, BATCH>(A, C, S, sm, t + 2);
+  } else {
+    static_assert(U == 1, "rings of three rows");
+    auto turn = [](auto* ring) {  // row r moves to the place of row r - 1, that one to r - 2's, that one to r - 3's
+      const auto t = ring[0];
+      ring[0] = ring[1];
+      ring[1] = ring[2];
+      ring[2] = t;
+    };
+    turn(S.cf);
+    turn(S.dux);
+    turn(S.suy);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      turn(S.w[q].T);
+      turn(S.w[q].w);
+      turn(S.w[q].e);
+    }
+  }
 }
 
 // Walk of strip sx, segment sg (rows [sg L, sg L + L)) of one domain by one warp.
-template <bool VEC, bool BATCH>
+// U: rows per pass of the loop.  U = 1 runs every row through the one general
+// body: five times less code, and a third more instructions (the rings move).
+template <int U, bool VEC, bool BATCH>
 __device__ __forceinline__ void energy_pair(const StepArgs& A, PairShared& sm, int L, int sx, int sg, int part, int s,
                                             int nsub) {
   PairCtx C;
@@ -407,17 +429,17 @@ __device__ __forceinline__ void energy_pair(const StepArgs& A, PairShared& sm, i
   S.ux = S.uy = S.uyS = S.qS = S.eh = S.el = z;
   const int t0 = C.ys - 4;
 #pragma unroll
-  for (int n = 0; n < EP_PF; ++n) pair_fetch<VEC>(A, C, sm, t0 + n * EP_U);
-  for (int t = t0; t < C.ye + 4; t += EP_U) {
-    // this group's rows (every lane's copies) are complete; the next group's slots
+  for (int n = 0; n < EP_PF / U; ++n) pair_fetch<U, VEC>(A, C, sm, t0 + n * U);
+  for (int t = t0; t < C.ye + 4; t += U) {
+    // this group's rows (every lane's copies) are complete; the fetched group's slots
     // hold rows that nothing reads any more
-    cp_async_wait<EP_PF - 1>();
+    cp_async_wait<EP_PF / U - 1>();
     __syncwarp();
-    pair_fetch<VEC>(A, C, sm, t + EP_PF * EP_U);
-    if (pair_bnd(A, t))
-      pair_group<true, VEC, BATCH>(A, C, S, sm, t);
+    pair_fetch<U, VEC>(A, C, sm, t + EP_PF);
+    if (U == 1 || pair_bnd<U>(A, t))
+      pair_group<U, true, VEC, BATCH>(A, C, S, sm, t);
     else
-      pair_group<false, VEC, BATCH>(A, C, S, sm, t);
+      pair_group<U, false, VEC, BATCH>(A, C, S, sm, t);
   }
   cp_async_wait<0>();  // none left in flight at exit
   // the warp's partials: q_bottom, q_top, q_interface, sensible energy
@@ -440,20 +462,22 @@ __device__ __forceinline__ void energy_pair(const StepArgs& A, PairShared& sm, i
 
 // One warp per CTA: everything that selects a branch or a row is then uniform
 // by construction and stays out of the vector registers.
+template <int U>
 __global__ void __launch_bounds__(32, EP_CTAS) k_energy_pair(const __grid_constant__ StepArgs A, int L, int s, int nsub) {
   __shared__ __align__(16) PairShared sm;
   // 16-byte prefetch pieces and 8-byte stores where the rows allow them
   if ((A.nx & 3) == 0)
-    energy_pair<true, false>(A, sm, L, blockIdx.x, blockIdx.y, blockIdx.y * gridDim.x + blockIdx.x, s, nsub);
+    energy_pair<U, true, false>(A, sm, L, blockIdx.x, blockIdx.y, blockIdx.y * gridDim.x + blockIdx.x, s, nsub);
   else
-    energy_pair<false, false>(A, sm, L, blockIdx.x, blockIdx.y, blockIdx.y * gridDim.x + blockIdx.x, s, nsub);
+    energy_pair<U, false, false>(A, sm, L, blockIdx.x, blockIdx.y, blockIdx.y * gridDim.x + blockIdx.x, s, nsub);
 }
 
+template <int U>
 __global__ void __launch_bounds__(32, EP_CTAS) k_energy_pair_batch(const __grid_constant__ StepArgs P,
-                                                                const DomArgs* __restrict__ desc,
-                                                                const int2* __restrict__ blk,
-                                                                const int* __restrict__ active, int L, int s,
-                                                                int nsub) {
+                                                                   const DomArgs* __restrict__ desc,
+                                                                   const int2* __restrict__ blk,
+                                                                   const int* __restrict__ active, int L, int s,
+                                                                   int nsub) {
   __shared__ __align__(16) PairShared sm;
   const int2 bl = blk[blockIdx.x];
   if (!active[bl.x]) return;
@@ -462,9 +486,9 @@ __global__ void __launch_bounds__(32, EP_CTAS) k_energy_pair_batch(const __grid_
   const int local = bl.y;
   const int strips = (A.nx + EP_OUT - 1) / EP_OUT;
   if ((A.nx & 3) == 0)
-    energy_pair<true, true>(A, sm, L, local % strips, local / strips, local, s, nsub);
+    energy_pair<U, true, true>(A, sm, L, local % strips, local / strips, local, s, nsub);
   else
-    energy_pair<false, true>(A, sm, L, local % strips, local / strips, local, s, nsub);
+    energy_pair<U, false, true>(A, sm, L, local % strips, local / strips, local, s, nsub);
 }
 
 }  // namespace hlb
