@@ -58,7 +58,7 @@ Offsets param_offsets(const Dims& d) {
 size_t al(size_t n) { return (n + 63) & ~(size_t)63; }  // 256-byte aligned float counts
 
 struct Acts {  // workspace offsets (floats)
-  size_t z1, a1, z2, a2, z3, a3, h0, z4, a4, z5, a5, y, dy, dz5, dz4, dh0, dz3, dz2, dz1, loss, total;
+  size_t z1, a1, z2, a2, z3, a3, h0, z4, a4, z5, a5, y, dy, dz5, dz4, dh0, dz3, dz2, dz1, loss, part, total;
 };
 
 Acts act_offsets(const Dims& d, int B) {
@@ -85,7 +85,8 @@ Acts act_offsets(const Dims& d, int B) {
   a.dz3 = p; p += al(n3);
   a.dz2 = p; p += al(n2);
   a.dz1 = p; p += al(n1);
-  a.loss = p; p += al(2);
+  a.loss = p; p += al(2 * (size_t)B);  // the fused path: one pair per sample
+  a.part = p; p += al((size_t)B * param_offsets(d).F1);  // and the convolutions' partial gradients
   a.total = p;
   return a;
 }
@@ -313,6 +314,412 @@ __global__ void k_adam(long long n, float* __restrict__ p, const float* __restri
   }
 }
 
+// ------------------------------------------------- one CTA per sample
+// Forward pass, loss and data gradients of one sample in one CTA, with every
+// activation in shared memory, for the framework's kernel size and stride (K = 5,
+// S = 2) and networks that fit.  The layer-by-layer kernels above take any other
+// sizes; on a batch of 64 their 21 launches cost more than their arithmetic (243
+// MFLOP), and the convolutions' inner loops read every operand from L1.  Here a
+// thread forms eight output channels of one position from one input value and two
+// broadcast 16-byte weight loads per tap, so that the FP32 pipe and shared memory
+// are about equally busy.  The convolutions' weight gradients leave the CTA as
+// per-sample partials (in the layout of the parameters), which k_sample_grads adds
+// in the order of the samples together with the linear layers' products.
+constexpr int SK = 5, SS = 2, ST = 512;  // taps, stride, threads
+
+struct SampleLayout {  // shared-memory offsets (floats); rows of odd length
+  int s1, s2, s3, p2, p3;
+  int x, w1, wt2, wt3, a1, a2, a3, d2, d1, h0, a4, a5, z, g, total;
+};
+
+__host__ __device__ inline SampleLayout sample_layout(const Dims& d, bool train) {
+  SampleLayout L;
+  L.s1 = d.L1 | 1;
+  L.s2 = d.L2 | 1;
+  L.s3 = d.L3 | 1;
+  L.p2 = (d.C2 + 7) & ~7;
+  L.p3 = (d.C3 + 7) & ~7;
+  int o = 0;
+  auto take = [&](int n) {
+    const int at = o;
+    o += (n + 3) & ~3;
+    return at;
+  };
+  L.wt2 = take(d.C1 * SK * L.p2);
+  L.wt3 = take(d.C2 * SK * L.p3);
+  L.x = take(d.L0);
+  L.w1 = take(d.C1 * SK);
+  L.a1 = take(d.C1 * L.s1);
+  L.a2 = take(d.C2 * L.s2);
+  L.a3 = take(d.C3 * L.s3);
+  L.d2 = train ? take(d.C2 * L.s2) : o;
+  L.d1 = train ? take(d.C1 * L.s1) : o;
+  L.h0 = take(d.C3 + d.NS);
+  L.a4 = take(d.H);
+  L.a5 = take(d.H);
+  L.z = take(d.NOUT > d.H ? d.NOUT : d.H);
+  L.g = train ? take(ST > 2 * d.H ? ST : 2 * d.H) : o;
+  L.total = o;
+  return L;
+}
+
+constexpr int SAMPLE_SMEM = 200 * 1024;
+
+bool sample_fits(const Dims& d, bool train) {
+  return d.K == SK && d.S == SS && (size_t)sample_layout(d, train).total * sizeof(float) <= SAMPLE_SMEM;
+}
+
+// W (Cout, Cin, 5) -> wt[(c 5 + k) Cp + o], zero-padded to Cp channels
+__device__ __forceinline__ void stage_weights(const float* __restrict__ W, int Cin, int Cout, int Cp, float* wt) {
+  const int n = Cin * SK * Cp;
+  for (int e = threadIdx.x; e < n; e += ST) {
+    const int o = e % Cp, ck = e / Cp;
+    wt[e] = o < Cout ? __ldg(W + (long long)o * Cin * SK + ck) : 0.f;
+  }
+}
+
+// out = relu(bias + conv(in)): eight channels of one position per thread and pass
+__device__ __forceinline__ void sample_conv(const float* in, int Cin, int sin, const float* wt, int Cp,
+                                            const float* __restrict__ bias, int Cout, int Lout, float* out, int sout) {
+  const int n = (Cp / 8) * Lout;
+  for (int e = threadIdx.x; e < n; e += ST) {
+    const int t = e % Lout, o0 = 8 * (e / Lout);
+    float s[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) s[j] = o0 + j < Cout ? __ldg(bias + o0 + j) : 0.f;
+    const float* x = in + SS * t;
+    const float* w = wt + o0;
+    for (int c = 0; c < Cin; ++c) {
+#pragma unroll
+      for (int k = 0; k < SK; ++k) {
+        const float v = x[c * sin + k];
+        const float4 w0 = *reinterpret_cast<const float4*>(w + (c * SK + k) * Cp);
+        const float4 w1 = *reinterpret_cast<const float4*>(w + (c * SK + k) * Cp + 4);
+        s[0] += w0.x * v, s[1] += w0.y * v, s[2] += w0.z * v, s[3] += w0.w * v;
+        s[4] += w1.x * v, s[5] += w1.y * v, s[6] += w1.z * v, s[7] += w1.w * v;
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      if (o0 + j < Cout) out[(o0 + j) * sout + t] = fmaxf(s[j], 0.f);
+  }
+}
+
+// din[c,u] = (act[c,u] > 0) sum over (o, k, t) with 2 t + k = u of W[o,c,k] dz[o,t]
+__device__ __forceinline__ void sample_conv_bwd(const float* dz, int Cout, int Lout, int sout, const float* wt, int Cp,
+                                                const float* act, int Cin, int Lin, int sin, float* din) {
+  const int half = (Lin + 1) / 2, n = Cin * 2 * half;
+  for (int e = threadIdx.x; e < n; e += ST) {
+    const int m = e % half, par = (e / half) & 1, c = e / (2 * half), u = 2 * m + par;
+    if (u >= Lin) continue;
+    float s = 0.f;
+    for (int k = par; k < SK; k += 2) {
+      const int t = m - (k - par) / 2;
+      if (t < 0 || t >= Lout) continue;
+      const float* w = wt + (c * SK + k) * Cp;
+      int o = 0;
+      for (; o + 4 <= Cout; o += 4) {
+        const float4 w4 = *reinterpret_cast<const float4*>(w + o);
+        s += w4.x * dz[o * sout + t];
+        s += w4.y * dz[(o + 1) * sout + t];
+        s += w4.z * dz[(o + 2) * sout + t];
+        s += w4.w * dz[(o + 3) * sout + t];
+      }
+      for (; o < Cout; ++o) s += w[o] * dz[o * sout + t];
+    }
+    din[c * sin + u] = act[c * sin + u] > 0.f ? s : 0.f;
+  }
+}
+
+// gW[o,c,k] = sum_t dz[o,t] in[c,2t+k] for two output channels o and one c per thread
+__device__ __forceinline__ void sample_conv_w(const float* dz, int Cout, int Lout, int sout, const float* in, int Cin,
+                                              int sin, float* __restrict__ gW) {
+  const int n = ((Cout + 1) / 2) * Cin;
+  for (int e = threadIdx.x; e < n; e += ST) {
+    const int c = e % Cin, o = 2 * (e / Cin), o1 = o + 1 < Cout ? o + 1 : o;
+    float a[SK] = {0.f, 0.f, 0.f, 0.f, 0.f}, b[SK] = {0.f, 0.f, 0.f, 0.f, 0.f};
+    const float* x = in + c * sin;
+    float x0 = x[0], x1 = x[1], x2 = x[2];
+    for (int t = 0; t < Lout; ++t) {
+      const float x3 = x[2 * t + 3], x4 = x[2 * t + 4];
+      const float da = dz[o * sout + t], db = dz[o1 * sout + t];
+      a[0] += da * x0, a[1] += da * x1, a[2] += da * x2, a[3] += da * x3, a[4] += da * x4;
+      b[0] += db * x0, b[1] += db * x1, b[2] += db * x2, b[3] += db * x3, b[4] += db * x4;
+      x0 = x2, x1 = x3, x2 = x4;
+    }
+#pragma unroll
+    for (int k = 0; k < SK; ++k) {
+      gW[((long long)o * Cin + c) * SK + k] = a[k];
+      if (o1 != o) gW[((long long)o1 * Cin + c) * SK + k] = b[k];
+    }
+  }
+}
+
+// gb[o] = sum_t dz[o,t], one warp per channel
+__device__ __forceinline__ void sample_bias_grad(const float* dz, int C, int L, int s, float* __restrict__ gb) {
+  const int lane = threadIdx.x & 31;
+  for (int o = threadIdx.x >> 5; o < C; o += ST / 32) {
+    float v = 0.f;
+    for (int t = lane; t < L; t += 32) v += dz[o * s + t];
+#pragma unroll
+    for (int q = 16; q > 0; q >>= 1) v += __shfl_xor_sync(0xffffffffu, v, q);
+    if (lane == 0) gb[o] = v;
+  }
+}
+
+// z[n] = bias[n] + sum_k F[n,k] x[k], four rows per warp at a time (relu optional)
+__device__ __forceinline__ void sample_linear(const float* __restrict__ F, const float* __restrict__ bias,
+                                              const float* x, int Nin, int Nout, float* z, bool relu) {
+  const int lane = threadIdx.x & 31;
+  const bool vec = (Nin & 3) == 0 && ((uintptr_t)F & 15) == 0;  // (x is 16-byte aligned)
+  for (int n0 = 4 * (threadIdx.x >> 5); n0 < Nout; n0 += 4 * (ST / 32)) {
+    float s[4] = {0.f, 0.f, 0.f, 0.f};
+    const float* row[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) row[j] = F + (long long)min(n0 + j, Nout - 1) * Nin;
+    if (vec) {
+      for (int k = 4 * lane; k < Nin; k += 128) {
+        const float4 v = *reinterpret_cast<const float4*>(x + k);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const float4 w = __ldg(reinterpret_cast<const float4*>(row[j] + k));
+          s[j] += w.x * v.x + w.y * v.y + (w.z * v.z + w.w * v.w);
+        }
+      }
+    } else {
+      for (int k = lane; k < Nin; k += 32) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) s[j] += __ldg(row[j] + k) * x[k];
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+#pragma unroll
+      for (int q = 16; q > 0; q >>= 1) s[j] += __shfl_xor_sync(0xffffffffu, s[j], q);
+      if (lane == j && n0 + j < Nout) {
+        const float v = s[j] + __ldg(bias + n0 + j);
+        z[n0 + j] = relu ? fmaxf(v, 0.f) : v;
+      }
+    }
+  }
+}
+
+// dx[k] = (act[k] > 0, if act) sum_n dz[n] F[n,k]; g: scratch of max(ST, 2 Nin) floats.
+// Columns across threads (coalesced rows of F), the rows dealt to groups of threads.
+__device__ __forceinline__ void sample_linear_bwd(const float* __restrict__ F, const float* dz, int Nout, int Nin,
+                                                  const float* act, float* dx, float* g) {
+  const int ng = Nin < ST ? ST / Nin : 1;
+  for (int e = threadIdx.x; e < ng * Nin; e += ST) {
+    const int k = e % Nin, part = e / Nin;
+    float s = 0.f;
+#pragma unroll 8
+    for (int n = part; n < Nout; n += ng) s += dz[n] * __ldg(F + (long long)n * Nin + k);
+    g[e] = s;
+  }
+  __syncthreads();
+  for (int k = threadIdx.x; k < Nin; k += ST) {
+    float s = 0.f;
+    for (int part = 0; part < ng; ++part) s += g[part * Nin + k];
+    dx[k] = act && !(act[k] > 0.f) ? 0.f : s;
+  }
+  __syncthreads();
+}
+
+struct SampleOut {  // what k_sample leaves for k_sample_grads (all per sample)
+  float *h0, *a4, *dz4, *a5, *dz5, *dy, *part, *loss;
+};
+
+template <bool TRAIN>
+__global__ void __launch_bounds__(ST, 1) k_sample(const Dims d, const Offsets o, const float* __restrict__ P,
+                                                  const float* __restrict__ hist, const float* __restrict__ scal,
+                                                  float* __restrict__ y, const float* __restrict__ target,
+                                                  const int* __restrict__ label, const SampleOut out) {
+  extern __shared__ __align__(16) float sm[];
+  const SampleLayout L = sample_layout(d, TRAIN);
+  const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, W0 = d.C3 + d.NS;
+  float *x = sm + L.x, *w1 = sm + L.w1, *wt2 = sm + L.wt2, *wt3 = sm + L.wt3, *a1 = sm + L.a1, *a2 = sm + L.a2,
+        *a3 = sm + L.a3, *h0 = sm + L.h0, *a4 = sm + L.a4, *a5 = sm + L.a5, *z = sm + L.z;
+  for (int e = tid; e < d.L0; e += ST) x[e] = __ldg(hist + (long long)b * d.L0 + e);
+  for (int e = tid; e < d.C1 * SK; e += ST) w1[e] = __ldg(P + o.W1 + e);
+  stage_weights(P + o.W2, d.C1, d.C2, L.p2, wt2);
+  stage_weights(P + o.W3, d.C2, d.C3, L.p3, wt3);
+  __syncthreads();
+  for (int e = tid; e < d.C1 * d.L1; e += ST) {
+    const int t = e % d.L1, c = e / d.L1;
+    float s = __ldg(P + o.b1 + c);
+#pragma unroll
+    for (int k = 0; k < SK; ++k) s += w1[c * SK + k] * x[SS * t + k];
+    a1[c * L.s1 + t] = fmaxf(s, 0.f);
+  }
+  __syncthreads();
+  sample_conv(a1, d.C1, L.s1, wt2, L.p2, P + o.b2, d.C2, d.L2, a2, L.s2);
+  __syncthreads();
+  sample_conv(a2, d.C2, L.s2, wt3, L.p3, P + o.b3, d.C3, d.L3, a3, L.s3);
+  __syncthreads();
+  for (int c = warp; c < d.C3; c += ST / 32) {
+    float s = 0.f;
+    for (int t = lane; t < d.L3; t += 32) s += a3[c * L.s3 + t];
+#pragma unroll
+    for (int q = 16; q > 0; q >>= 1) s += __shfl_xor_sync(0xffffffffu, s, q);
+    if (lane == 0) h0[c] = s / (float)d.L3;
+  }
+  for (int j = tid; j < d.NS; j += ST) h0[d.C3 + j] = scal[(long long)b * d.NS + j];
+  __syncthreads();
+  sample_linear(P + o.F1, P + o.c1, h0, W0, d.H, a4, true);
+  __syncthreads();
+  sample_linear(P + o.F2, P + o.c2, a4, d.H, d.H, a5, true);
+  __syncthreads();
+  sample_linear(P + o.F3, P + o.c3, a5, d.H, d.NOUT, z, false);
+  __syncthreads();
+  if constexpr (!TRAIN) {
+    for (int n = tid; n < d.NOUT; n += ST) y[(long long)b * d.NOUT + n] = z[n];
+    return;
+  }
+  float *d2 = sm + L.d2, *d1 = sm + L.d1, *g = sm + L.g;
+  for (int k = tid; k < W0; k += ST) out.h0[(long long)b * W0 + k] = h0[k];
+  for (int k = tid; k < d.H; k += ST) {
+    out.a4[(long long)b * d.H + k] = a4[k];
+    out.a5[(long long)b * d.H + k] = a5[k];
+  }
+  if (tid == 0) {  // loss terms and dL/dy of the sample, y in place
+    const float invB = 1.f / (float)gridDim.x;
+    const float r = z[0] - target[b];
+    float m = z[1];
+    for (int q = 2; q < d.NOUT; ++q) m = fmaxf(m, z[q]);
+    float se = 0.f;
+    for (int q = 1; q < d.NOUT; ++q) se += expf(z[q] - m);
+    const int lb = label[b];
+    out.loss[2 * b] = r * r;
+    out.loss[2 * b + 1] = logf(se) + m - z[1 + lb];
+    z[0] = 2.f * r * invB;
+    for (int q = 1; q < d.NOUT; ++q) z[q] = (expf(z[q] - m) / se - (q - 1 == lb ? 1.f : 0.f)) * invB;
+    for (int q = 0; q < d.NOUT; ++q) out.dy[(long long)b * d.NOUT + q] = z[q];
+  }
+  __syncthreads();
+  sample_linear_bwd(P + o.F3, z, d.NOUT, d.H, a5, a5, g);  // a5 becomes dz5
+  sample_linear_bwd(P + o.F2, a5, d.H, d.H, a4, a4, g);    // a4 becomes dz4
+  for (int k = tid; k < d.H; k += ST) {
+    out.dz5[(long long)b * d.H + k] = a5[k];
+    out.dz4[(long long)b * d.H + k] = a4[k];
+  }
+  sample_linear_bwd(P + o.F1, a4, d.H, W0, nullptr, h0, g);
+  for (int e = tid; e < d.C3 * d.L3; e += ST) {  // a3 becomes dz3
+    const int t = e % d.L3, c = e / d.L3;
+    float* p = a3 + c * L.s3 + t;
+    *p = *p > 0.f ? h0[c] / (float)d.L3 : 0.f;
+  }
+  __syncthreads();
+  sample_conv_bwd(a3, d.C3, d.L3, L.s3, wt3, L.p3, a2, d.C2, d.L2, L.s2, d2);
+  float* part = out.part + (long long)b * o.F1;
+  sample_conv_w(a3, d.C3, d.L3, L.s3, a2, d.C2, L.s2, part + o.W3);
+  sample_bias_grad(a3, d.C3, d.L3, L.s3, part + o.b3);
+  __syncthreads();
+  sample_conv_bwd(d2, d.C2, d.L2, L.s2, wt2, L.p2, a1, d.C1, d.L1, L.s1, d1);
+  sample_conv_w(d2, d.C2, d.L2, L.s2, a1, d.C1, L.s1, part + o.W2);
+  sample_bias_grad(d2, d.C2, d.L2, L.s2, part + o.b2);
+  __syncthreads();
+  for (int c = warp; c < d.C1; c += ST / 32) {
+    float s[SK + 1] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    for (int t = lane; t < d.L1; t += 32) {
+      const float v = d1[c * L.s1 + t];
+#pragma unroll
+      for (int k = 0; k < SK; ++k) s[k] += v * x[SS * t + k];
+      s[SK] += v;
+    }
+#pragma unroll
+    for (int k = 0; k <= SK; ++k) {
+#pragma unroll
+      for (int q = 16; q > 0; q >>= 1) s[k] += __shfl_xor_sync(0xffffffffu, s[k], q);
+      if (lane == 0) part[k < SK ? o.W1 + c * SK + k : o.b1 + c] = s[k];
+    }
+  }
+}
+
+// One 16 x 16 tile of dF[n,k] = sum_b dz[b,n] x[b,k] (column Nin: the bias gradient)
+__device__ __forceinline__ void linear_grad_tile(const float* __restrict__ dz, const float* __restrict__ x, int B,
+                                                 int Nout, int Nin, int bx, int by, float* __restrict__ dF,
+                                                 float* __restrict__ dc) {
+  __shared__ float ds[TL][TL + 1], xs[TL][TL + 1];
+  const int tx = threadIdx.x % TL, ty = threadIdx.x / TL;
+  const int n = by * TL + ty, k = bx * TL + tx;
+  float s = 0.f;
+  for (int b0 = 0; b0 < B; b0 += TL) {
+    // rows of both operands are read along their columns
+    const int b = b0 + ty, nd = by * TL + tx;
+    ds[tx][ty] = (b < B && nd < Nout) ? dz[(long long)b * Nout + nd] : 0.f;
+    xs[ty][tx] = b < B && k <= Nin ? (k < Nin ? x[(long long)b * Nin + k] : 1.f) : 0.f;
+    __syncthreads();
+#pragma unroll
+    for (int bb = 0; bb < TL; ++bb) s += ds[ty][bb] * xs[bb][tx];
+    __syncthreads();
+  }
+  if (n < Nout && k <= Nin) (k < Nin ? dF[(long long)n * Nin + k] : dc[n]) = s;
+}
+
+// Parameter gradients from the samples' results: tiles of the three linear layers,
+// the sums of the convolutions' partials, and the loss (last block).
+__global__ void __launch_bounds__(256) k_sample_grads(const Dims d, const Offsets o, int B, const SampleOut w,
+                                                      float* __restrict__ G, float* __restrict__ loss) {
+  const int W0 = d.C3 + d.NS, th = (d.H + TL - 1) / TL, th1 = (d.H + TL) / TL, tw1 = (W0 + TL) / TL,
+            to = (d.NOUT + TL - 1) / TL;
+  int id = blockIdx.x;
+  if (id < th1 * th) {
+    linear_grad_tile(w.dz5, w.a4, B, d.H, d.H, id % th1, id / th1, G + o.F2, G + o.c2);
+    return;
+  }
+  id -= th1 * th;
+  if (id < tw1 * th) {
+    linear_grad_tile(w.dz4, w.h0, B, d.H, W0, id % tw1, id / tw1, G + o.F1, G + o.c1);
+    return;
+  }
+  id -= tw1 * th;
+  if (id < th1 * to) {
+    linear_grad_tile(w.dy, w.a5, B, d.NOUT, d.H, id % th1, id / th1, G + o.F3, G + o.c3);
+    return;
+  }
+  id -= th1 * to;
+  const int n = (int)o.F1, nb = (n + 255) / 256;
+  if (id < nb) {
+    const int e = id * 256 + threadIdx.x;
+    if (e >= n) return;
+    float s = 0.f;
+#pragma unroll 8
+    for (int b = 0; b < B; ++b) s += w.part[(long long)b * n + e];
+    G[e] = s;
+    return;
+  }
+  float mse = 0.f, ce = 0.f;
+  for (int b = threadIdx.x; b < B; b += 256) {
+    mse += w.loss[2 * b];
+    ce += w.loss[2 * b + 1];
+  }
+  mse = block_sum<256>(mse);
+  __syncthreads();
+  ce = block_sum<256>(ce);
+  if (threadIdx.x == 0) {
+    loss[0] = mse / (float)B;
+    loss[1] = ce / (float)B;
+  }
+}
+
+int sample_grad_blocks(const Dims& d, const Offsets& o) {
+  const int W0 = d.C3 + d.NS, th = (d.H + TL - 1) / TL, th1 = (d.H + TL) / TL, tw1 = (W0 + TL) / TL,
+            to = (d.NOUT + TL - 1) / TL;
+  return th1 * th + tw1 * th + th1 * to + ((int)o.F1 + 255) / 256 + 1;
+}
+
+// Launch k_sample on B samples (its shared memory is allowed on every call:
+// nothing is kept from one call to the next).
+template <bool TRAIN>
+hlb_status launch_sample(const Dims& d, const Offsets& o, const float* P, const float* hist, const float* scal, int B,
+                         float* y, const float* target, const int* label, const SampleOut& out, cudaStream_t s) {
+  const size_t smem = (size_t)sample_layout(d, TRAIN).total * sizeof(float);
+  if (cudaFuncSetAttribute(k_sample<TRAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+    return HLB_ECUDA;
+  k_sample<TRAIN><<<B, ST, smem, s>>>(d, o, P, hist, scal, y, target, label, out);
+  return HLB_OK;
+}
+
 int grid_for(long long n) {
   long long g = (n + 255) / 256;
   return (int)(g > 4096 ? 4096 : (g < 1 ? 1 : g));
@@ -381,6 +788,11 @@ hlb_status hlb_sur_forward(const hlb_sur_config* c, const float* d_params, const
   const Acts A = act_offsets(d, B);
   float* w = (float*)d_ws;
   cudaStream_t s = (cudaStream_t)stream;
+  if (sample_fits(d, false)) {
+    const hlb_status st = launch_sample<false>(d, o, d_params, d_hist, d_scal, B, d_out, nullptr, nullptr, SampleOut{}, s);
+    if (st != HLB_OK) return st;
+    return cudaGetLastError() == cudaSuccess ? HLB_OK : HLB_ECUDA;
+  }
   forward(d, o, A, d_params, d_hist, d_scal, B, w, s);
   if (cudaMemcpyAsync(d_out, w + A.y, sizeof(float) * (size_t)B * d.NOUT, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
     return HLB_ECUDA;
@@ -401,6 +813,13 @@ hlb_status hlb_sur_loss_grad(const hlb_sur_config* c, const float* d_params, con
   const float* P = d_params;
   float* G = d_grad;
   cudaStream_t s = (cudaStream_t)stream;
+  if (sample_fits(d, true)) {
+    const SampleOut out = {w + A.h0, w + A.a4, w + A.dz4, w + A.a5, w + A.dz5, w + A.dy, w + A.part, w + A.loss};
+    const hlb_status st = launch_sample<true>(d, o, P, d_hist, d_scal, B, nullptr, d_target, d_label, out, s);
+    if (st != HLB_OK) return st;
+    k_sample_grads<<<sample_grad_blocks(d, o), 256, 0, s>>>(d, o, B, out, G, d_loss);
+    return cudaGetLastError() == cudaSuccess ? HLB_OK : HLB_ECUDA;
+  }
   forward(d, o, A, P, d_hist, d_scal, B, w, s);
   k_loss<<<1, 256, 0, s>>>(w + A.y, B, d.NOUT, d_target, d_label, w + A.dy, w + A.loss);
   const dim3 blk(TL, TL);
