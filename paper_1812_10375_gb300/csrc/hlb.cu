@@ -412,6 +412,7 @@ struct hlb_domain {
   float* ftop[2] = {nullptr, nullptr};
   double* partials = nullptr;
   DevState* state = nullptr;
+  DevState* pin = nullptr;  // page-locked host copy of the record (hlb_diag)
   double* hist = nullptr;
   // N > 1 (Eq. 27): rho^n, u_x^n, u_y^n of the step, a T buffer and the
   // sub-steps' per-block partials
@@ -560,7 +561,7 @@ hlb_status launch_step(hlb_domain* d) {
     float* rho = d->mom;
     float* ux = d->mom + N;
     float* uy = d->mom + 2 * N;
-    k_read<<<INIT_BLOCKS, 256, 0, d->stream>>>(a, d->T[d->parity], 0, rho, ux, uy);
+    k_read<<<INIT_BLOCKS, 256, 0, d->stream>>>(a, d->T[d->parity], 0, rho, ux, uy, nullptr, nullptr);
     float* Tcur = d->T[d->parity ^ 1];
     float* Tother = d->Tscr;
     const int nsub = d->p.n_sub;
@@ -637,6 +638,27 @@ hlb_status set_fields_at(hlb_domain* d, const float* d_rho, const float* d_T, in
   d->fields_set = true;
   d->host_flags = 0;
   return HLB_OK;
+}
+
+// Page-locked host memory for n diagnostics records; null (hlb_diag then copies
+// through pageable memory) if there is none to be had.  Both calls run in the
+// relaxed capture mode: they touch no stream, and another thread's capture of its
+// own stream stays valid.
+struct RelaxedCapture {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+DevState* pinned_records(int n) {
+  RelaxedCapture relaxed;
+  void* p = nullptr;
+  if (cudaHostAlloc(&p, (size_t)n * sizeof(DevState), cudaHostAllocDefault) == cudaSuccess) return (DevState*)p;
+  cudaGetLastError();
+  return nullptr;
+}
+void free_records(DevState* p) {
+  RelaxedCapture relaxed;
+  if (p) cudaFreeHost(p);
 }
 
 hlb_status init_domain(hlb_domain* d, const hlb_params* p, char* ws, cudaStream_t stream) {
@@ -1383,6 +1405,7 @@ hlb_status hlb_init(hlb_domain** out, const hlb_params* p, void* d_workspace, si
     delete d;
     return st;
   }
+  d->pin = pinned_records(1);
   *out = d;
   return HLB_OK;
 }
@@ -1456,24 +1479,24 @@ hlb_status hlb_read(hlb_domain* d, float* d_rho, float* d_ux, float* d_uy, float
   const int cur = d->parity;
   StepArgs a = args_for(d, cur ^ 1);
   // args_for(cur ^ 1) has f_out = f[cur] (the current populations)
-  if (d_rho || d_ux || d_uy) {
+  if (d_rho || d_ux || d_uy || d_T) {
     const float* Tn = d->T[cur ^ 1];  // T^n: the temperature the last step started from
     k_read<<<INIT_BLOCKS, 256, 0, d->stream>>>(a, d->steps == 0 ? d->T[cur] : Tn, d->steps == 0 ? 1 : 0, d_rho,
-                                                d_ux, d_uy);
-  }
-  if (d_T) {
-    if (cudaMemcpyAsync(d_T, d->T[cur], sizeof(float) * (size_t)d->p.nx * d->p.ny, cudaMemcpyDeviceToDevice,
-                        d->stream) != cudaSuccess)
-      return HLB_ECUDA;
+                                                d_ux, d_uy, d->T[cur], d_T);
   }
   return cudaGetLastError() == cudaSuccess ? HLB_OK : HLB_ECUDA;
 }
 
 hlb_status hlb_diag(hlb_domain* d, hlb_diag_record* out) {
   if (!d || !out) return HLB_EINVAL;
-  DevState s;
-  if (cudaMemcpyAsync(&s, d->state, sizeof(s), cudaMemcpyDeviceToHost, d->stream) != cudaSuccess) return HLB_ECUDA;
+  // into page-locked memory the copy is one operation on the stream; through
+  // pageable memory it is staged by the driver
+  DevState pageable;
+  DevState* const rec = d->pin ? d->pin : &pageable;
+  if (cudaMemcpyAsync(rec, d->state, sizeof(DevState), cudaMemcpyDeviceToHost, d->stream) != cudaSuccess)
+    return HLB_ECUDA;
   if (cudaStreamSynchronize(d->stream) != cudaSuccess) return HLB_ECUDA;
+  const DevState& s = *rec;
   out->step = s.step;
   out->mass = s.mass;
   out->energy = s.energy;
@@ -1502,6 +1525,7 @@ hlb_status hlb_reset_timeavg(hlb_domain* d) {
 hlb_status hlb_destroy(hlb_domain* d) {
   if (!d) return HLB_EINVAL;
   drop_graph(d);
+  free_records(d->pin);
   delete d;
   return HLB_OK;
 }
@@ -1591,6 +1615,8 @@ hlb_status hlb_batch_init(hlb_batch** out, int n, const hlb_params* p, void* d_w
     delete b;
     return st;
   }
+  DevState* const pin = pinned_records(n);
+  for (int i = 0; pin && i < n; ++i) b->dom[i].pin = pin + i;
   *out = b;
   return HLB_OK;
 }
@@ -1744,6 +1770,7 @@ hlb_status hlb_batch_destroy(hlb_batch* b) {
   if (!b) return HLB_EINVAL;
   batch_drop_graph(b);
   for (auto& d : b->dom) drop_graph(&d);
+  free_records(b->dom[0].pin);
   delete b;
   return HLB_OK;
 }

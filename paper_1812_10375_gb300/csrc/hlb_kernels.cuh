@@ -966,15 +966,37 @@ __global__ void k_init_state(const double* __restrict__ partials, int nblk, DevS
 
 // rho^n and u^n from the stored post-collision populations: collision keeps
 // mass and leaves sum_i e_i f*_i = rho u + F/2 (Eqs. 2, 5, 8), so
-// u = (sum e f* - F/2) / rho with F recomputed from rho^n and T^n.
+// u = (sum e f* - F/2) / rho with F recomputed from rho^n and T^n; and a copy of
+// T^{n+1}, for which the call needs no second operation on the stream.  Without
+// u a cell needs only its own populations (no neighbours' psi): 36 B read
+// instead of nine times that through L1, and no division by nx.
 __global__ void __launch_bounds__(256) k_read(const StepArgs A, const float* __restrict__ Tn, int zero_u,
-                                              float* rho_out, float* ux_out, float* uy_out) {
+                                              float* rho_out, float* ux_out, float* uy_out,
+                                              const float* __restrict__ T_new, float* T_copy) {
   const Geo g = make_geo(A);
   const long long N = A.plane;  // population plane stride (>= nx ny)
   const long long NC = (long long)A.nx * A.ny;
+  const long long first = blockIdx.x * (long long)blockDim.x + threadIdx.x, step = (long long)gridDim.x * blockDim.x;
+  if (T_copy)
+    for (long long c = first; c < NC; c += step) T_copy[c] = __ldg(T_new + c);
+  if (!ux_out && !uy_out) {
+    if (!rho_out) return;
+    const long long lo = (long long)A.W * A.nx, hi = g.top_wall ? NC - A.nx : NC;
+    for (long long c = first; c < NC; c += step) {
+      float r = 0.f;
+      if (c >= lo && c < hi) {
+        float f[9];
+#pragma unroll
+        for (int q = 0; q < 9; ++q) f[q] = A.f_out[q * N + c];
+        r = A.rho_ref + sum9(f);
+      }
+      rho_out[c] = r;
+    }
+    return;
+  }
   const float rho_ave = (float)A.state->rho_ave_prev;
-  for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < NC; c += (long long)gridDim.x * blockDim.x) {
-    const int y = (int)(c / A.nx), x = (int)(c % A.nx);
+  for (long long c = first; c < NC; c += step) {
+    const int y = (int)((unsigned)c / (unsigned)A.nx), x = (int)((unsigned)c % (unsigned)A.nx);  // (NC < 2^28)
     if (g.solid_row(y)) {
       if (rho_out) rho_out[c] = 0.f;
       if (ux_out) ux_out[c] = 0.f;
