@@ -629,9 +629,9 @@ bool variant_ok(const hlb_domain* d, int v) {
 hlb_status set_fields_at(hlb_domain* d, const float* d_rho, const float* d_T, int par) {
   if (!d || !d_rho || !d_T) return HLB_EINVAL;
   StepArgs a = args_for(d, par);
-  k_init<<<INIT_BLOCKS, 256, 0, d->stream>>>(a, d_rho, d_T, d->f[par], d->T[par], d->ftop[0], d->ftop[1]);
-  k_init<<<INIT_BLOCKS, 256, 0, d->stream>>>(a, d_rho, d_T, d->f[par ^ 1], d->T[par ^ 1], nullptr, nullptr);
-  k_init_state<<<1, 32, 0, d->stream>>>(d->partials, INIT_BLOCKS, d->state, 1.0 / (double)d->n_fluid);
+  k_init<<<INIT_BLOCKS, 256, 0, d->stream>>>(a, d_rho, d_T, d->f[par], d->T[par], d->f[par ^ 1], d->T[par ^ 1],
+                                             d->ftop[0], d->ftop[1]);
+  k_init_state<<<1, 256, 0, d->stream>>>(d->partials, INIT_BLOCKS, d->state, 1.0 / (double)d->n_fluid);
   if (cudaGetLastError() != cudaSuccess) return HLB_ECUDA;
   d->parity = par;
   d->steps = 0;

@@ -905,26 +905,28 @@ __global__ void __launch_bounds__(256) k_reduce_batch(const ReduceArgs* __restri
 }
 
 // Initial state: f* = rest equilibrium w_i rho (deviation form), T with the
-// Dirichlet rows set, the convective-outlet memory, and per-block fluid mass.
+// Dirichlet rows set, in both buffer sets; the convective-outlet memory, and
+// per-block fluid mass.
 __global__ void __launch_bounds__(256) k_init(const StepArgs A, const float* __restrict__ rho0,
                                               const float* __restrict__ T0, float* __restrict__ f,
-                                              float* __restrict__ T, float* __restrict__ ftop_a,
+                                              float* __restrict__ T, float* __restrict__ f_b,
+                                              float* __restrict__ T_b, float* __restrict__ ftop_a,
                                               float* __restrict__ ftop_b) {
   const Geo g = make_geo(A);
   const long long N = A.plane;  // population plane stride (>= nx ny)
   const long long NC = (long long)A.nx * A.ny;
   double mass = 0.0;
   for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < NC; c += (long long)gridDim.x * blockDim.x) {
-    const int y = (int)(c / A.nx), x = (int)(c % A.nx);
+    const int y = (int)((unsigned)c / (unsigned)A.nx), x = (int)((unsigned)c % (unsigned)A.nx);  // (NC < 2^28)
     const bool solid = g.solid_row(y);
     const float d = solid ? 0.f : rho0[c] - A.rho_ref;
     const float w[9] = {4.f / 9.f, 1.f / 9.f, 1.f / 9.f, 1.f / 9.f, 1.f / 9.f,
                         1.f / 36.f, 1.f / 36.f, 1.f / 36.f, 1.f / 36.f};
 #pragma unroll
-    for (int q = 0; q < 9; ++q) f[q * N + c] = solid ? 0.f : w[q] * d;
-    T[c] = g.dirichlet_row(y) ? (y == 0 ? A.T_bottom : A.T_top) : T0[c];
+    for (int q = 0; q < 9; ++q) f[q * N + c] = f_b[q * N + c] = solid ? 0.f : w[q] * d;
+    T[c] = T_b[c] = g.dirichlet_row(y) ? (y == 0 ? A.T_bottom : A.T_top) : T0[c];
     if (!solid) mass += (double)rho0[c];
-    if (y == A.ny - 1 && ftop_a) {
+    if (y == A.ny - 1) {
       ftop_a[x] = w[4] * d;
       ftop_a[A.nx + x] = w[7] * d;
       ftop_a[2 * A.nx + x] = w[8] * d;
@@ -944,10 +946,17 @@ __global__ void __launch_bounds__(256) k_init(const StepArgs A, const float* __r
   }
 }
 
-__global__ void k_init_state(const double* __restrict__ partials, int nblk, DevState* st, double inv_nfluid) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
+__global__ void __launch_bounds__(256) k_init_state(const double* __restrict__ partials, int nblk, DevState* st,
+                                                    double inv_nfluid) {
+  __shared__ double s_red[8];
+  double v = 0.0;
+  for (int b = threadIdx.x; b < nblk; b += 256) v += partials[(long long)b * NPART + P_MASS];
+  v = warp_sum(v);
+  if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  if (threadIdx.x == 0) {
     double m = 0.0;
-    for (int b = 0; b < nblk; ++b) m += partials[(long long)b * NPART + P_MASS];
+    for (int q = 0; q < 8; ++q) m += s_red[q];
     st->rho_ave = m * inv_nfluid;
     st->rho_ave_prev = st->rho_ave;
     st->U = 0.0;
