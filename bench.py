@@ -45,8 +45,8 @@ ENERGY_BYTES_FLUID = 4 + 12 + 4
 ENERGY_BYTES_SOLID = 8
 KIND_SPLIT, KIND_FUSED, KIND_MARCH = 0, 1, 2
 
-KERNEL_SOURCES = ("hlb_internal.cuh", "hlb_kernels.cuh", "hlb_march.cuh", "hlb_split.cuh",
-                  "hlb_energy_walk.cuh")  # step kernels' device code
+KERNEL_SOURCES = ("hlb_internal.cuh", "hlb_kernels.cuh", "hlb_march.cuh", "hlb_split.cuh", "hlb_energy_walk.cuh",
+                  "hlb_pair.cuh", "hlb_energy_pair.cuh")  # step kernels' device code
 
 
 def kernel_source_hash() -> str:
@@ -391,14 +391,18 @@ def run_ours(args):
     ms_per_step, value = aggregate(elapsed_ms, cells, args.steps, dist)
     kern_avg_ms = sum(kern_ms) / len(kern_ms)
     kernels = None
+    # variant 0 walks its rows by one warp, the other split variants by two
+    step_names = kernel_name(variants[chosen], kind, erows).split("+")
+    if chosen == 0:
+        step_names[-1] = "k_energy_pair_batch"
     if kind == KIND_SPLIT:
         flow_ms = sum(ev_b[k].elapsed_time(ev_f[k]) for k in range(n_ev)) / n_ev
         en_ms = sum(ev_f[k].elapsed_time(ev_a[k]) for k in range(n_ev)) / n_ev
         fb = FLOW_BYTES_FLUID * n_fluid
         eb = ENERGY_BYTES_FLUID * n_fluid + ENERGY_BYTES_SOLID * n_solid
         kernels = {"k_flow_batch": {"ms": flow_ms, "bytes_per_launch": fb, "gbs": fb / (flow_ms * 1e-3) / 1e9},
-                   energy_kernel_name(erows): {"ms": en_ms, "bytes_per_launch": eb,
-                                               "gbs": eb / (en_ms * 1e-3) / 1e9}}
+                   step_names[-1]: {"ms": en_ms, "bytes_per_launch": eb,
+                                    "gbs": eb / (en_ms * 1e-3) / 1e9}}
     diag0 = batch.diag(0, check_flags=False)
 
     # end to end through the public API with host buffers (skipped by --quick,
@@ -434,7 +438,7 @@ def run_ours(args):
                                 "tuning_ms_per_step": [round(m, 4) for m in tune_ms]}},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak, "traffic": traffic,
-                         "kernel": kernel_name(variants[chosen], kind, erows), "bytes_per_launch": bytes_per_step,
+                         "kernel": "+".join(step_names), "bytes_per_launch": bytes_per_step,
                          "bytes_note": "the step's algorithmic bytes (80 B per fluid cell, 8 B per solid cell) "
                                        "over the step kernels' time per step",
                          "kernel_ms": kern_avg_ms, "peak_source": peak_src, "per_kernel": kernels},

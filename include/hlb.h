@@ -320,9 +320,11 @@ hlb_status hlb_batch_destroy(hlb_batch* b);
 /* ------------------------------------------------------------- autotuning
  * The step is compiled in three kinds (hlb_variant_kind):
  *  - HLB_KIND_SPLIT: a flow kernel over tiles of 64 columns by a few fluid-row
- *    heights, then N energy sub-step kernels: a row-walking kernel over strips
- *    of 56 columns and segments of 96, 64 or 32 rows, or a tiled one over
- *    56 x 24 tiles (finite-volume scheme; the default for it);
+ *    heights, then N energy sub-step kernels over strips of 56 columns: a walk
+ *    up the rows by one warp (variant 0, the default for the finite-volume
+ *    scheme: its segments and its flow tile are sized by the lattices, and the
+ *    heights it reports are those of large ones) or by two warps (segments of 96
+ *    or 64 rows), or a tiled kernel over 56 x 24 tiles;
  *  - HLB_KIND_FUSED: one fused step kernel over 52-column tiles of a few
  *    heights, with 256 or 512 threads per CTA (the default for the isotropic
  *    scheme, which only this kind runs);

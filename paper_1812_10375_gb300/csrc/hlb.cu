@@ -189,11 +189,12 @@ static_assert(EW_OUT == EN_TX && EP_OUT == EN_TX, "walk strips and energy tiles 
 
 // Segment rows of the one-warp energy walk for n lattices (strips of EP_OUT
 // columns, ny rows each): the smallest height at which every segment is resident at
-// once.  A warp's rows follow one another (0.30 us a row alone, 0.58 us with two
+// once.  A warp's rows follow one another (about 0.3 us a row alone, 0.6 us with two
 // warps on a scheduler), so short segments win until the chip is full; beyond that a
-// second wave costs more than taller segments: the 32-domain sweep took 0.0594 ms
-// with 1,142 segments of 86 rows, 0.070 with 901 of 112 and 0.072 with 1,815 of 54;
-// 14 lattices of 400 x 600 0.047 ms with 1,120 of 60, 0.055 with 1,792 of 38.
+// second wave costs more than taller segments.  The energy kernel on the 32-domain
+// sweep, by segments (an earlier form of it, 10% faster throughout): 1,142 of 86 rows
+// 0.059 ms, 901 of 112 0.070, 1,815 of 54 0.072; on 14 lattices of 400 x 600: 1,120 of
+// 60 rows 0.047 ms, 1,792 of 38 0.055.
 int walk_rows(int n, const int* strips, const int* ny) {
   auto segments = [&](int L) {
     long long w = 0;

@@ -16,17 +16,21 @@
 // rounding: both columns of a packed instruction round on their own, so the new
 // temperature is the same bit for bit.
 //
-// Why this shape: the update is bound by instruction issue, not by memory (20 B
-// per cell).  Two columns per lane make every arithmetic instruction a packed
-// one, the neighbouring columns come from two shuffles per row and field, shared
-// memory holds the prefetched input rows only, and no barrier is needed.  The
-// loop is unrolled by three, not four: the rings' indices become constants and
-// its 12 KB of instructions still fit the instruction cache nearest to a
-// scheduler (four rows: 0.7 warps per issue waited for instructions; one row, its
-// rings moved in registers: 30% more instructions).  Against the two-warp walk
-// with one column per thread, on the 32-domain sweep (5.0 M cells): 0.0594 against
-// 0.0795 ms; one 400 x 400 lattice: 0.0131 against 0.052 ms, mostly by its shorter
-// segments (walk_rows in hlb.cu).
+// Why this shape: the update is bound by instruction issue and by the latency of a
+// row's dependent stages, not by memory (20 B per cell).  Two columns per lane make
+// most arithmetic instructions packed ones, the neighbouring columns come from two
+// shuffles per row and field, shared memory holds the prefetched input rows only,
+// and no barrier is needed.  One warp per CTA keeps everything that selects a branch
+// or a row uniform, out of the vector registers (384-thread CTAs spilled 1 KB).  The
+// loop is unrolled by three, not four: the rings' indices become constants and its
+// instructions still fit the cache nearest to a scheduler (four rows: 0.7 warps per
+// issue waited for instructions).  Segments of up to 12 rows take the one-row form
+// (pair_short in hlb.cu).  Twelve warps per SM instead of eight (168 registers)
+// spilled and were slower on one lattice and no faster on the sweep.
+// Against the two-warp walk with one column per thread, the kernel alone: 32-domain
+// sweep (4.9 M cells, 1,142 segments of 86 rows) 0.066 against 0.079 ms; 14 lattices
+// of 400 x 600 0.052 against 0.059; 400 x 400 about 0.009 against 0.052, mostly by its
+// shorter segments (walk_rows in hlb.cu).
 #pragma once
 #include "hlb_pair.cuh"
 #include "hlb_split.cuh"

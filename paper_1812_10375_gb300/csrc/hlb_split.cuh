@@ -7,19 +7,24 @@
 //   Peng-Robinson EOS at T^n (Eqs. 7, 28) -> F = F_m + F_ads + F_b (Eqs. 6, 9,
 //   10) -> u (Eq. 5) -> MRT collision with Li's forcing (Eqs. 2-4, 8).  It
 //   writes the post-collision populations and rho^n, u^n for the energy update.
-//   A tile is 64 columns by TY fluid rows; psi of its cells and of a one-cell
-//   ring around it goes through shared memory (the ring's populations are
-//   pulled again by this CTA, from L2).  Each thread keeps the pulled
-//   populations of its own cells in registers between the psi pass and the
-//   collision, so every population is loaded once and stored once.
-// k_energy (N launches per step): one RK4 sub-step (Eq. 18, dt = 1/N) of the
-//   energy equation (Eq. 17) with the finite-volume harmonic face
-//   conductivities of Eqs. (22)-(26), on rho^n and u^n held over the
-//   sub-steps.  A 56 x 24 tile in a 64 x 32 frame; stage k is evaluated on
-//   ring 4 - k of the tile.  Each thread owns a run of 8 rows of one frame
-//   column: the per-cell coefficients of Eq. (17) (four face terms with the
-//   axis part of the advection folded in, two diagonal advection terms, the
-//   two latent-heat coefficients, rho cv) and the run's stage values stay in
+//   A tile is 64 columns by TY fluid rows (24, or fewer on lattices that do not
+//   fill the chip); psi of its cells and of a one-cell ring around it goes
+//   through shared memory (the ring's populations are pulled again by this CTA,
+//   from L2).  After the barrier each thread pulls its own cells again, which
+//   costs L2 reads but leaves 64 registers and four CTAs per SM.  At 4.7 TB/s of
+//   its own traffic on the 32-domain sweep the kernel is bound by L2 and DRAM
+//   latency, not by issue: 5% more integer instructions or 15% fewer L2 reads (the
+//   populations stashed in shared memory) left its time as it was or longer.
+// k_energy_pair (hlb_energy_pair.cuh; N launches per step): one RK4 sub-step (Eq. 18,
+//   dt = 1/N) of the energy equation (Eq. 17) with the finite-volume harmonic
+//   face conductivities of Eqs. (22)-(26), on rho^n and u^n held over the
+//   sub-steps, one warp per strip of columns and segment of rows.
+// k_energy_walk, k_energy (selectable variants): the same sub-step by two warps per
+//   strip with barriers, and in 56 x 24 tiles of a 64 x 32 frame.  In a tile stage
+//   k is evaluated on ring 4 - k; each thread owns a run of 8 rows of one frame
+//   column: the per-cell coefficients of Eq. (17) (four face terms with the axis
+//   part of the advection folded in, two diagonal advection terms, the two
+//   latent-heat coefficients, rho cv) and the run's stage values stay in
 //   registers; shared memory carries only what neighbouring threads read (the
 //   stage values, u and lambda).
 // Both kernels write per-tile partial sums (flow: fluid mass, first-fluid-row
