@@ -183,8 +183,10 @@ hlb_status hlb_set_nucleation_sites(hlb_domain* d, int n, const hlb_site* h_site
 /* Advance nsteps coupled steps (asynchronous on the handle's stream).
  * Repeated calls reuse a captured CUDA graph of 16 steps.  A step of the split
  * form (the default for HLB_DIFF_FV) is a flow kernel, N energy sub-step
- * kernels and an FP64 reduction kernel; a step of a fused variant is the fused
- * step kernel and the reduction (see the autotuning section). */
+ * kernels and an FP64 reduction kernel, which on small lattices is part of the
+ * next step's flow kernel but for a call's (and a graph's) last step; a step of a
+ * fused variant is the fused step kernel and the reduction (see the autotuning
+ * section). */
 hlb_status hlb_step(hlb_domain* d, int nsteps);
 
 /* Fields after the last step: rho^n, u^n (the step's pre-collision moments,

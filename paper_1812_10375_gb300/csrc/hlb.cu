@@ -21,6 +21,7 @@ using namespace hlb;
 namespace {
 
 constexpr int NUM_SMS = 152;
+constexpr int HIST_CAP = 1 << 16;  // wall-flux history entries kept per domain
 constexpr int TILE_X = TILE_W;  // 52 output columns in a 64-wide frame
 
 // Compiled variants of the fused step kernel (tile height, threads per CTA).
@@ -62,6 +63,8 @@ struct FlowKernel {
   void (*launch_single)(dim3, size_t, cudaStream_t, const StepArgs&);
   void (*launch_batch)(int, size_t, cudaStream_t, const StepArgs&, const DomArgs*, const int2*, const int*,
                        const float2*);
+  // a chained step, with the reduction arguments of the step before; may be null
+  void (*launch_chain)(dim3, size_t, cudaStream_t, const StepArgs&, const SplitReduceArgs&);
 };
 struct FlowVariant {
   int fk;      // flow kernel (index into FLOW_KERNELS), or -1: by flow_kernel_for()
@@ -87,6 +90,21 @@ template <int TY, int NTH, int MINB, bool RP>
 void launch_flow_batch(int blocks, size_t smem, cudaStream_t s, const StepArgs& phys, const DomArgs* desc,
                        const int2* blk, const int* act, const float2* lag) {
   k_flow_batch<TY, NTH, MINB, RP><<<blocks, NTH, smem, s>>>(phys, desc, blk, act, lag);
+}
+template <int TY, int NTH, int MINB, bool RP>
+void launch_flow_chain(dim3 grid, size_t smem, cudaStream_t s, const StepArgs& a, const SplitReduceArgs& r) {
+  grid.y += 1;
+  if (r.nf <= CHAIN_FEW)
+    k_flow_chain<TY, NTH, MINB, RP, CHAIN_FEW><<<grid, NTH, smem, s>>>(a, r, HIST_CAP);
+  else
+    k_flow_chain<TY, NTH, MINB, RP, CHAIN_PARTS><<<grid, NTH, smem, s>>>(a, r, HIST_CAP);
+}
+template <int TY, int NTH, int MINB, bool RP>
+constexpr auto flow_chain() -> decltype(FlowKernel::launch_chain) {
+  if constexpr (TY <= CHAIN_TY && RP)
+    return launch_flow_chain<TY, NTH, MINB, RP>;
+  else
+    return nullptr;
 }
 template <int R, int NPH, int MINB>
 void launch_energy_single(dim3 grid, cudaStream_t s, const StepArgs& a, int sub, int nsub, int) {
@@ -128,7 +146,7 @@ void launch_pair_batch(int blocks, cudaStream_t s, const StepArgs& phys, const D
 #define HLB_FLOW_ENTRY(TY, NTH, MINB, RP)                                                                        \
   FlowKernel{TY, NTH, flow_smem_bytes<TY>(), (const void*)k_flow<TY, NTH, MINB, RP>,                             \
              (const void*)k_flow_batch<TY, NTH, MINB, RP>, launch_flow_single<TY, NTH, MINB, RP>,                \
-             launch_flow_batch<TY, NTH, MINB, RP>},
+             launch_flow_batch<TY, NTH, MINB, RP>, flow_chain<TY, NTH, MINB, RP>()},
 const FlowKernel FLOW_KERNELS[] = {HLB_FLOW_KERNELS(HLB_FLOW_ENTRY)};
 #define HLB_SPLIT_TILE(FK, ER, ENPH, EMINB)                                                                      \
   FlowVariant{FK, 0, ER, (const void*)k_energy<ER, ENPH, EMINB>, (const void*)k_energy_batch<ER, ENPH, EMINB>,   \
@@ -212,8 +230,12 @@ int walk_rows(int n, const int* strips, const int* ny) {
   }
   return lo;
 }
+size_t align_up(size_t v) { return (v + 255) & ~(size_t)255; }
 size_t flow_part_slots(int nx, int ny, int W, int top_bc) {
   return (size_t)((nx + FL_TX - 1) / FL_TX) * ((fluid_rows_of(ny, W, top_bc) + MIN_FLOW_TY - 1) / MIN_FLOW_TY);
+}
+size_t flow_part_bytes(const hlb_params* p) {
+  return align_up(flow_part_slots(p->nx, p->ny, p->wall_rows, p->top_bc) * NFPART * sizeof(double));
 }
 // Flow kernel for n lattices (tiles to a row of tiles, fluid rows): the shortest tile
 // whose CTAs are all resident at once (four per SM), else the 24-row one.  A thread
@@ -232,11 +254,9 @@ int flow_kernel_for(int n, const int* tx, const int* rows) {
   return best;
 }
 constexpr int GRAPH_STEPS = 16;     // steps per captured graph (even: buffers return to parity 0)
-constexpr int HIST_CAP = 1 << 16;   // wall-flux history entries kept per domain
 constexpr int INIT_BLOCKS = 304;
 constexpr int MAX_SUB = 64;  // largest N of Eq. (27)
 
-size_t align_up(size_t v) { return (v + 255) & ~(size_t)255; }
 
 // ------------------------------------------------------------ Peng-Robinson
 // Eq. (28) written in the specific volume v = 1/rho:
@@ -422,7 +442,7 @@ struct hlb_domain {
   double* subpart = nullptr;
   dim3 sub_grid;
   // split step: per-tile partials of the flow and energy kernels, energy grid
-  double* fpart = nullptr;
+  double* fpart[2] = {nullptr, nullptr};  // of chained steps by buffer parity, else the first
   double* epart = nullptr;
   dim3 egrid;
   int erows = 64;  // segment rows of the one-warp energy walk
@@ -478,7 +498,7 @@ Layout layout_of(const hlb_params* p) {
   L.hist = o;     o += align_up(HIST_CAP * sizeof(double));
   // rho^n, u_x^n, u_y^n of the step and a T plane for sub-steps
   L.mom = o;      o += align_up(4 * N * sizeof(float));
-  L.fpart = o;    o += align_up(flow_part_slots(p->nx, p->ny, p->wall_rows, p->top_bc) * NFPART * sizeof(double));
+  L.fpart = o;    o += 2 * flow_part_bytes(p);
   const dim3 eg = energy_grid_of(p->nx, p->ny);
   L.epart = o;    o += align_up((size_t)eg.x * eg.y * NEPART * sizeof(double));
   L.sub = o;
@@ -506,12 +526,13 @@ StepArgs args_for(hlb_domain* d, int par) {
   return a;
 }
 
-// The reduction's view of domain d under its split variant.
-SplitReduceArgs reduce_args_of(const hlb_domain* d) {
+// The reduction's view of domain d under its split variant, for the flow partials of
+// set `part`.
+SplitReduceArgs reduce_args_of(const hlb_domain* d, int part = 0) {
   const FlowVariant& fv = FLOWS[is_split(d->variant) ? d->variant : 0];
   const int ty = flow_kernel_of(d).ty, rows = fv.erows(d->erows);
   SplitReduceArgs r;
-  r.fpart = d->fpart;
+  r.fpart = d->fpart[part];
   r.epart = d->epart;
   r.state = d->state;
   r.hist = d->hist;
@@ -527,25 +548,39 @@ SplitReduceArgs reduce_args_of(const hlb_domain* d) {
   return r;
 }
 
+// Whether the steps of one call are chained (hlb_split.cuh).
+bool chains(const hlb_domain* d) {
+  return flow_kernel_of(d).launch_chain && (long long)d->grid.x * d->grid.y <= CHAIN_PARTS;
+}
+
 // One step of the split form: the flow kernel, N energy sub-steps, the reduction.
-hlb_status launch_split_step(hlb_domain* d, cudaEvent_t after_flow = nullptr, cudaEvent_t after_energy = nullptr) {
-  const StepArgs a = args_for(d, d->parity);
+// first, last: in the steps of one call or graph; between chained steps the
+// reduction is part of the next flow kernel.
+hlb_status launch_split_step(hlb_domain* d, bool first, bool last, cudaEvent_t after_flow = nullptr,
+                             cudaEvent_t after_energy = nullptr) {
+  StepArgs a = args_for(d, d->parity);
   const FlowVariant& fv = FLOWS[d->variant];
   const FlowKernel& fl = flow_kernel_of(d);
-  fl.launch_single(d->grid, fl.smem, d->stream, a);
+  const bool chain = chains(d);
+  const int part = chain ? d->parity : 0;
+  a.fpart = d->fpart[part];
+  if (chain && !first)
+    fl.launch_chain(d->grid, fl.smem, d->stream, a, reduce_args_of(d, part ^ 1));
+  else
+    fl.launch_single(d->grid, fl.smem, d->stream, a);
   if (after_flow && cudaEventRecord(after_flow, d->stream) != cudaSuccess) return HLB_ECUDA;
   const int nsub = d->p.n_sub;
   for (int s = 1; s <= nsub; ++s) fv.energy_single(d->egrid, d->stream, a, s, nsub, d->erows);
   if (after_energy && cudaEventRecord(after_energy, d->stream) != cudaSuccess) return HLB_ECUDA;
-  k_reduce_split<<<1, 256, 0, d->stream>>>(reduce_args_of(d), HIST_CAP);
+  if (last || !chain) k_reduce_split<<<1, 256, 0, d->stream>>>(reduce_args_of(d, part), HIST_CAP);
   if (cudaGetLastError() != cudaSuccess) return HLB_ECUDA;
   d->parity ^= 1;
   d->steps += 1;
   return HLB_OK;
 }
 
-hlb_status launch_step(hlb_domain* d) {
-  if (is_split(d->variant)) return launch_split_step(d);
+hlb_status launch_step(hlb_domain* d, bool first = true, bool last = true) {
+  if (is_split(d->variant)) return launch_split_step(d, first, last);
   const StepArgs a = args_for(d, d->parity);
   if (is_march(d->variant)) {
     k_march<<<d->grid, march_row_stride(d->p.nx), march_smem(d->p.nx), d->stream>>>(a, march_seg(d->variant));
@@ -600,7 +635,7 @@ hlb_status build_graph(hlb_domain* d) {
   if (cudaStreamBeginCapture(d->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return HLB_ECUDA;
   const long long s0 = d->steps;
   hlb_status st = HLB_OK;
-  for (int k = 0; k < GRAPH_STEPS && st == HLB_OK; ++k) st = launch_step(d);
+  for (int k = 0; k < GRAPH_STEPS && st == HLB_OK; ++k) st = launch_step(d, k == 0, k == GRAPH_STEPS - 1);
   const cudaError_t e = cudaStreamEndCapture(d->stream, &g);
   d->steps = s0;
   d->parity = 0;
@@ -694,7 +729,8 @@ hlb_status init_domain(hlb_domain* d, const hlb_params* p, char* ws, cudaStream_
   d->hist = (double*)(ws + L.hist);
   d->mom = (float*)(ws + L.mom);
   d->Tscr = d->mom + 3 * N;
-  d->fpart = (double*)(ws + L.fpart);
+  d->fpart[0] = (double*)(ws + L.fpart);
+  d->fpart[1] = (double*)(ws + L.fpart + flow_part_bytes(p));
   d->epart = (double*)(ws + L.epart);
   if (q.n_sub > 1) {
     d->subpart = (double*)(ws + L.sub);
@@ -758,7 +794,7 @@ hlb_status init_domain(hlb_domain* d, const hlb_params* p, char* ws, cudaStream_
   a.state = d->state;
   a.mom = d->mom;
   a.T_scr = d->Tscr;
-  a.fpart = d->fpart;
+  a.fpart = d->fpart[0];
   a.epart = d->epart;
 
   for (const FlowKernel& k : FLOW_KERNELS) {
@@ -1457,6 +1493,7 @@ hlb_status hlb_step(hlb_domain* d, int nsteps) {
   if (d->host_flags) return HLB_ESTATE;
   hlb_status st = HLB_OK;
   const bool graphs = d->stream != nullptr;
+  bool first = true;
   while (nsteps > 0 && st == HLB_OK) {
     if (graphs && d->parity == 0 && nsteps >= GRAPH_STEPS) {
       if (!d->graph) {
@@ -1467,8 +1504,11 @@ hlb_status hlb_step(hlb_domain* d, int nsteps) {
       d->steps += GRAPH_STEPS;
       nsteps -= GRAPH_STEPS;
     } else {
-      st = launch_step(d);
       nsteps -= 1;
+      // a chain ends with the call, or where a graph follows
+      const bool last = nsteps == 0 || (graphs && d->parity == 1 && nsteps >= GRAPH_STEPS);
+      st = launch_step(d, first, last);
+      first = last;
     }
   }
   return st;

@@ -137,10 +137,135 @@ __device__ __forceinline__ void block_partials(float (&ah)[NQ], float (&al)[NQ],
   }
 }
 
+// ------------------------------------------------------------- reduction
+// Where a domain's partial sums lie: the flow tiles' (nf, tx tiles to a row of
+// tiles) and the energy blocks' (ne, strips to a row of blocks).  Every block has
+// mass or energy; the other quantities come from one row of blocks each: the
+// vapour count of row W from the first row of flow tiles, u_y of row ny - 2 from
+// the tiles at ut0, q_bottom from the first row of energy blocks, q_interface and
+// q_top from the blocks at qi0 and qt0.
+struct SplitReduceArgs {
+  const double* fpart;
+  const double* epart;
+  DevState* state;
+  double* hist;
+  int nf, ne, tx, strips, ut0, qi0, qt0;
+  double inv_nfluid, inv_nx;
+};
+
+// Sums the flow and energy kernels' partials of one domain (one CTA) and updates
+// the record: lagged mean density (Eq. 9) and outlet velocity for the next
+// step, diagnostics, running sums, flux history.  The FP64 pipe (a warp's add takes
+// 16 cycles of an SM's) and the record's load latency bound it: mass and energy are
+// added in four-entry strides and folded by one warp each, the one-row quantities
+// by a warp each, and the record's old values are fetched before the sums.
+// One CTA adding seven sums of every partial took 8.5 us of a 33 us step of one
+// 400 x 400 lattice (912 partials); so ordered, 5.
+__device__ __forceinline__ void reduce_split_block(const SplitReduceArgs& r, int hist_cap, float2* lag) {
+  enum { R_MASS, R_ENERGY, R_VCOV, R_UTOP, R_QB, R_QT, R_QI, NR };
+  __shared__ double s_part[2][256];
+  __shared__ double s_sum[NR];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  DevState* const st = r.state;
+  DevState old;
+  if (tid == 0) old = *st;
+  double m = 0.0, e = 0.0;
+  for (int b = tid; b < r.nf; b += 256) m += r.fpart[(long long)b * NFPART + FP_MASS];
+  for (int b = tid; b < r.ne; b += 256) e += r.epart[(long long)b * NEPART + EP_E];
+  s_part[0][tid] = m;
+  s_part[1][tid] = e;
+  if (warp >= R_VCOV && warp < NR) {
+    const bool flow = warp <= R_UTOP;
+    const int n = flow ? r.tx : r.strips;
+    const int at = warp == R_UTOP ? r.ut0 : (warp == R_QT ? r.qt0 : (warp == R_QI ? r.qi0 : 0));
+    const int q = warp == R_VCOV ? FP_VCOV : (warp == R_UTOP ? FP_UTOP : (warp == R_QB ? EP_QB : (warp == R_QT ? EP_QT : EP_QI)));
+    const double* p = flow ? r.fpart : r.epart;
+    const int stride = flow ? NFPART : NEPART;
+    double v = 0.0;
+    if (at >= 0)
+      for (int b = lane; b < n; b += 32) v += p[(long long)(at + b) * stride + q];
+    v = warp_sum(v);
+    if (lane == 0) s_sum[warp] = v;
+  }
+  __syncthreads();
+  if (warp < 2) {
+    double v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = s_part[warp][lane + 32 * k];
+    const double t = warp_sum(((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7])));
+    if (lane == 0) s_sum[warp] = t;
+  }
+  __syncthreads();
+  if (tid == 0) {
+    const double rho_ave = s_sum[R_MASS] * r.inv_nfluid;
+    const double ut = s_sum[R_UTOP] * r.inv_nx;
+    const double U = ut > 0.0 ? ut : 0.0;
+    const double Uc = U > 0.0 ? U / (1.0 + U) : 0.0;
+    if (lag) *lag = make_float2((float)Uc, (float)rho_ave);
+    const double qb = s_sum[R_QB] * r.inv_nx, vcov = s_sum[R_VCOV] * r.inv_nx;
+    st->rho_ave_prev = old.rho_ave;
+    st->rho_ave = rho_ave;
+    st->u_top = ut;
+    st->U = U;
+    st->Uc = Uc;
+    st->step = old.step + 1;
+    st->mass = s_sum[R_MASS];
+    st->energy = s_sum[R_ENERGY];
+    st->q_bottom = qb;
+    st->q_top = s_sum[R_QT] * r.inv_nx;
+    st->q_interface = s_sum[R_QI] * r.inv_nx;
+    st->q_sum = old.q_sum + qb;
+    st->q_count = old.q_count + 1;
+    st->vcov = vcov;
+    st->vcov_sum = old.vcov_sum + vcov;
+    if (r.hist && old.hist_len < hist_cap) {
+      r.hist[old.hist_len] = qb;
+      st->hist_len = old.hist_len + 1;
+    }
+  }
+}
+
+// Chained steps: between two steps of one call the flow kernel of the second takes
+// the lagged scalars from the partials of the first, and one CTA beside its tiles
+// updates the record, instead of a launch between them that runs one CTA.
+// Every tile adds all partials (one warp, while the others pull), so the lattices
+// are those whose tiles are all resident at once, CHAIN_PARTS of them at most; a
+// batch's launch between the steps costs less than its tiles' sums (32 boiling
+// domains: 161 us a step, chained 165).  Whole steps before and after: 200 x 100 (96
+// tiles) 18.3 and 16.0 us, 256 x 200 (196) 18.8 and 17.4, 385 x 301 (518) 22.7 and
+// 19.9; with the few tiles' form the long one's 19 loads and adds are spared (200 x
+// 100: 16.9 with them).
+constexpr int CHAIN_PARTS = 608, CHAIN_FEW = 128;
+constexpr int CHAIN_TY = 16;  // the tallest tile that is compiled so
+
+// The lagged scalars after the step with reduction arguments r: x = U / (1 + U),
+// y = mean density.  One warp, adding in reduce_split_block's order, so that a step's
+// results do not depend on whether it is chained.  PARTS: the partials it has room
+// for; all loads are in flight together, and a form for few of them is the shorter.
+template <int PARTS>
+__device__ __forceinline__ float2 lag_from_partials(const SplitReduceArgs& r) {
+  const int lane = threadIdx.x & 31;
+  double u = 0.0, v[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+  if (r.ut0 >= 0)
+    for (int b = lane; b < r.tx; b += 32) u += r.fpart[(r.ut0 + b) * NFPART + FP_UTOP];
+#pragma unroll
+  for (int k = 0; k < PARTS / 32; ++k) {
+    const int b = lane + 32 * k;
+    const double p = b < r.nf ? r.fpart[b * NFPART + FP_MASS] : 0.0;
+    v[k & 7] = k < 8 ? p : v[k & 7] + p;
+  }
+  double m = (v[0] + v[1]) + (v[2] + v[3]);
+  if (PARTS > 128) m += (v[4] + v[5]) + (v[6] + v[7]);
+  const double mass = warp_sum(m), ut = warp_sum(u) * r.inv_nx;
+  return make_float2(ut > 0.0 ? (float)(ut / (1.0 + ut)) : 0.f, (float)(mass * r.inv_nfluid));
+}
+
 // ---------------------------------------------------------------- flow tile
-template <int TY, int NTH, bool INT, bool RP>
+// CH: a chained step, with room for CH partials of the step before (0: not chained);
+// prev: that step's reduction arguments (else null).
+template <int TY, int NTH, bool INT, bool RP, int CH = 0>
 __device__ __forceinline__ void flow_tile(const StepArgs& A, int bx, int by, int part, float* sPsi, float Uc,
-                                          float rho_ave) {
+                                          float rho_ave, const SplitReduceArgs* prev = nullptr) {
   constexpr int NPH = NTH / FL_TX;
   constexpr int CPT = TY / NPH;  // own cells per thread: a run of CPT rows of one column
   constexpr int NHALO = 2 * FL_FW + 2 * TY;
@@ -163,6 +288,19 @@ __device__ __forceinline__ void flow_tile(const StepArgs& A, int bx, int by, int
   const int NC = nx * ny;
   if (tid == 0) s_err = 0;
   int err = 0;
+  // tiles that reach the open top need U in pass 1, the others only the mean
+  // density, after the barrier
+  __shared__ float2 s_lag;
+  if constexpr (CH > 0) {
+    if (tid >= NTH - 32) {
+      const float2 l = lag_from_partials<CH>(*prev);
+      if (tid == NTH - 32) s_lag = l;
+    }
+    if constexpr (!INT) {
+      __syncthreads();
+      Uc = s_lag.x;
+    }
+  }
 
   // psi of a fluid node from its density and temperature (Eq. 7 with Eq. 28)
   auto psi_of = [&](float rho, float T) -> float {
@@ -248,6 +386,7 @@ __device__ __forceinline__ void flow_tile(const StepArgs& A, int bx, int by, int
     sPsi[(j + 1) * FL_FW + ii + 1] = ps;
   }
   __syncthreads();
+  if constexpr (CH > 0) rho_ave = s_lag.y;
 
   // ---- pass 2: forces, velocity, collision of the own cells
   float ah[NFPART], al[NFPART];
@@ -322,6 +461,25 @@ __global__ void __launch_bounds__(NTH, MINB) k_flow(const StepArgs A) {
     flow_tile<TY, NTH, true, RP>(A, blockIdx.x, blockIdx.y, part, sm, Uc, rho_ave);
   else
     flow_tile<TY, NTH, false, RP>(A, blockIdx.x, blockIdx.y, part, sm, Uc, rho_ave);
+}
+
+// The flow kernel of a chained step; r: the reduction arguments of the step before.
+// The first row of blocks is one that updates its record (the tiles do not read it).
+template <int TY, int NTH, int MINB, bool RP, int CH>
+__global__ void __launch_bounds__(NTH, MINB) k_flow_chain(const StepArgs A, const __grid_constant__ SplitReduceArgs r,
+                                                          int hist_cap) {
+  static_assert(NTH == 256, "the reduction takes 256 threads");
+  extern __shared__ float sm[];
+  if (blockIdx.y == 0) {
+    if (blockIdx.x == 0) reduce_split_block(r, hist_cap, nullptr);
+    return;
+  }
+  const int by = blockIdx.y - 1;
+  const int part = by * gridDim.x + blockIdx.x;
+  if (flow_interior(A, A.W + by * TY, TY))
+    flow_tile<TY, NTH, true, RP, CH>(A, blockIdx.x, by, part, sm, 0.f, 0.f, &r);
+  else
+    flow_tile<TY, NTH, false, RP, CH>(A, blockIdx.x, by, part, sm, 0.f, 0.f, &r);
 }
 
 // Loads the domain descriptor of block `b` into shared memory; returns false
@@ -805,94 +963,6 @@ __global__ void __launch_bounds__(64 * NPH, MINB) k_energy_batch(const StepArgs 
     energy_tile_int<R, NPH>(A, local % tx, by, local, sm, s, nsub);
   else
     energy_tile<R, NPH>(A, local % tx, by, local, sm, s, nsub);
-}
-
-// ------------------------------------------------------------- reduction
-// Where a domain's partial sums lie: the flow tiles' (nf, tx tiles to a row of
-// tiles) and the energy blocks' (ne, strips to a row of blocks).  Every block has
-// mass or energy; the other quantities come from one row of blocks each: the
-// vapour count of row W from the first row of flow tiles, u_y of row ny - 2 from
-// the tiles at ut0, q_bottom from the first row of energy blocks, q_interface and
-// q_top from the blocks at qi0 and qt0.
-struct SplitReduceArgs {
-  const double* fpart;
-  const double* epart;
-  DevState* state;
-  double* hist;
-  int nf, ne, tx, strips, ut0, qi0, qt0;
-  double inv_nfluid, inv_nx;
-};
-
-// Sums the flow and energy kernels' partials of one domain (one CTA) and updates
-// the record: lagged mean density (Eq. 9) and outlet velocity for the next
-// step, diagnostics, running sums, flux history.  The FP64 pipe (a warp's add takes
-// 16 cycles of an SM's) and the record's load latency bound it: mass and energy are
-// added in four-entry strides and folded by one warp each, the one-row quantities
-// by a warp each, and the record's old values are fetched before the sums.
-// One CTA adding seven sums of every partial took 8.5 us of a 33 us step of one
-// 400 x 400 lattice (912 partials); so ordered, 5.
-__device__ __forceinline__ void reduce_split_block(const SplitReduceArgs& r, int hist_cap, float2* lag) {
-  enum { R_MASS, R_ENERGY, R_VCOV, R_UTOP, R_QB, R_QT, R_QI, NR };
-  __shared__ double s_part[2][256];
-  __shared__ double s_sum[NR];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  DevState* const st = r.state;
-  DevState old;
-  if (tid == 0) old = *st;
-  double m = 0.0, e = 0.0;
-  for (int b = tid; b < r.nf; b += 256) m += r.fpart[(long long)b * NFPART + FP_MASS];
-  for (int b = tid; b < r.ne; b += 256) e += r.epart[(long long)b * NEPART + EP_E];
-  s_part[0][tid] = m;
-  s_part[1][tid] = e;
-  if (warp >= R_VCOV && warp < NR) {
-    const bool flow = warp <= R_UTOP;
-    const int n = flow ? r.tx : r.strips;
-    const int at = warp == R_UTOP ? r.ut0 : (warp == R_QT ? r.qt0 : (warp == R_QI ? r.qi0 : 0));
-    const int q = warp == R_VCOV ? FP_VCOV : (warp == R_UTOP ? FP_UTOP : (warp == R_QB ? EP_QB : (warp == R_QT ? EP_QT : EP_QI)));
-    const double* p = flow ? r.fpart : r.epart;
-    const int stride = flow ? NFPART : NEPART;
-    double v = 0.0;
-    if (at >= 0)
-      for (int b = lane; b < n; b += 32) v += p[(long long)(at + b) * stride + q];
-    v = warp_sum(v);
-    if (lane == 0) s_sum[warp] = v;
-  }
-  __syncthreads();
-  if (warp < 2) {
-    double v[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) v[k] = s_part[warp][lane + 32 * k];
-    const double t = warp_sum(((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7])));
-    if (lane == 0) s_sum[warp] = t;
-  }
-  __syncthreads();
-  if (tid == 0) {
-    const double rho_ave = s_sum[R_MASS] * r.inv_nfluid;
-    const double ut = s_sum[R_UTOP] * r.inv_nx;
-    const double U = ut > 0.0 ? ut : 0.0;
-    const double Uc = U > 0.0 ? U / (1.0 + U) : 0.0;
-    if (lag) *lag = make_float2((float)Uc, (float)rho_ave);
-    const double qb = s_sum[R_QB] * r.inv_nx, vcov = s_sum[R_VCOV] * r.inv_nx;
-    st->rho_ave_prev = old.rho_ave;
-    st->rho_ave = rho_ave;
-    st->u_top = ut;
-    st->U = U;
-    st->Uc = Uc;
-    st->step = old.step + 1;
-    st->mass = s_sum[R_MASS];
-    st->energy = s_sum[R_ENERGY];
-    st->q_bottom = qb;
-    st->q_top = s_sum[R_QT] * r.inv_nx;
-    st->q_interface = s_sum[R_QI] * r.inv_nx;
-    st->q_sum = old.q_sum + qb;
-    st->q_count = old.q_count + 1;
-    st->vcov = vcov;
-    st->vcov_sum = old.vcov_sum + vcov;
-    if (r.hist && old.hist_len < hist_cap) {
-      r.hist[old.hist_len] = qb;
-      st->hist_len = old.hist_len + 1;
-    }
-  }
 }
 
 __global__ void __launch_bounds__(256) k_reduce_split(const __grid_constant__ SplitReduceArgs r, int hist_cap) {
