@@ -760,13 +760,15 @@ int sample_grad_blocks(const Dims& d, const Offsets& o) {
   return th1 * th + tw1 * th + th1 * to + ((int)o.F1 + 255) / 256 + 1;
 }
 
-// Launch k_sample on B samples (its shared memory is allowed on every call:
-// nothing is kept from one call to the next).
+// Launch k_sample on B samples.  The shared memory a kernel may take is one value per
+// function and device, seen by every host thread: each call sets the most that any
+// network takes (sample_fits), so that no call lowers it between another thread's
+// setting and its launch.
 template <bool TRAIN>
 hlb_status launch_sample(const Dims& d, const Offsets& o, const float* P, const float* hist, const float* scal, int B,
                          float* y, const float* target, const int* label, const SampleOut& out, cudaStream_t s) {
   const size_t smem = (size_t)sample_layout(d, TRAIN).total * sizeof(float);
-  if (cudaFuncSetAttribute(k_sample<TRAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+  if (cudaFuncSetAttribute(k_sample<TRAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, SAMPLE_SMEM) != cudaSuccess)
     return HLB_ECUDA;
   k_sample<TRAIN><<<B, ST, smem, s>>>(d, o, P, hist, scal, y, target, label, out);
   return HLB_OK;
