@@ -57,6 +57,52 @@ Offsets param_offsets(const Dims& d) {
 
 size_t al(size_t n) { return (n + 63) & ~(size_t)63; }  // 256-byte aligned float counts
 
+// What the per-sample kernels (below) need of a network.
+constexpr int SK = 5, SS = 2, ST = 512;  // taps, stride, threads
+
+struct SampleLayout {  // shared-memory offsets (floats); rows of odd length
+  int s1, s2, s3, p2, p3;
+  int x, w1, wt2, wt3, a1, a2, a3, d2, d1, h0, a4, a5, z, g, total;
+};
+
+__host__ __device__ inline SampleLayout sample_layout(const Dims& d, bool train) {
+  SampleLayout L;
+  L.s1 = d.L1 | 1;
+  L.s2 = d.L2 | 1;
+  L.s3 = d.L3 | 1;
+  L.p2 = (d.C2 + 7) & ~7;
+  L.p3 = (d.C3 + 7) & ~7;
+  int o = 0;
+  auto take = [&](int n) {
+    const int at = o;
+    o += (n + 3) & ~3;
+    return at;
+  };
+  L.wt2 = take(d.C1 * SK * L.p2);
+  L.wt3 = take(d.C2 * SK * L.p3);
+  L.x = take(d.L0);
+  L.w1 = take(d.C1 * SK);
+  L.a1 = take(d.C1 * L.s1);
+  L.a2 = take(d.C2 * L.s2);
+  L.a3 = take(d.C3 * L.s3);
+  L.d2 = train ? take(d.C2 * L.s2) : o;
+  L.d1 = train ? take(d.C1 * L.s1) : o;
+  L.h0 = take(d.C3 + d.NS);
+  L.a4 = take(d.H);
+  L.a5 = take(d.H);
+  L.z = take(d.NOUT > d.H ? d.NOUT : d.H);
+  const int widest = d.H > d.C3 + d.NS ? d.H : d.C3 + d.NS;
+  L.g = train ? take(4 * ST > widest ? 4 * ST : widest) : o;
+  L.total = o;
+  return L;
+}
+
+constexpr int SAMPLE_SMEM = 200 * 1024;
+
+bool sample_fits(const Dims& d, bool train) {
+  return d.K == SK && d.S == SS && (size_t)sample_layout(d, train).total * sizeof(float) <= SAMPLE_SMEM;
+}
+
 struct Acts {  // workspace offsets (floats)
   size_t z1, a1, z2, a2, z3, a3, h0, z4, a4, z5, a5, y, dy, dz5, dz4, dh0, dz3, dz2, dz1, loss, part, total;
 };
@@ -85,8 +131,10 @@ Acts act_offsets(const Dims& d, int B) {
   a.dz3 = p; p += al(n3);
   a.dz2 = p; p += al(n2);
   a.dz1 = p; p += al(n1);
-  a.loss = p; p += al(2 * (size_t)B);  // the fused path: one pair per sample
-  a.part = p; p += al((size_t)B * param_offsets(d).F1);  // and the convolutions' partial gradients
+  // by samples: a pair of loss terms and the convolutions' partial gradients of each
+  const bool samples = sample_fits(d, true);
+  a.loss = p; p += al(samples ? 2 * (size_t)B : 2);
+  a.part = p; p += samples ? al((size_t)B * param_offsets(d).F1) : 0;
   a.total = p;
   return a;
 }
@@ -328,50 +376,6 @@ __global__ void k_adam(long long n, float* __restrict__ p, const float* __restri
 // network: a training step of 64 samples 317 -> 70 us (k_sample 55 of them: one CTA
 // on each of 64 SMs, bound by the latency of its dozen dependent phases), a forward
 // call of 96 samples 77 -> 27 us.
-constexpr int SK = 5, SS = 2, ST = 512;  // taps, stride, threads
-
-struct SampleLayout {  // shared-memory offsets (floats); rows of odd length
-  int s1, s2, s3, p2, p3;
-  int x, w1, wt2, wt3, a1, a2, a3, d2, d1, h0, a4, a5, z, g, total;
-};
-
-__host__ __device__ inline SampleLayout sample_layout(const Dims& d, bool train) {
-  SampleLayout L;
-  L.s1 = d.L1 | 1;
-  L.s2 = d.L2 | 1;
-  L.s3 = d.L3 | 1;
-  L.p2 = (d.C2 + 7) & ~7;
-  L.p3 = (d.C3 + 7) & ~7;
-  int o = 0;
-  auto take = [&](int n) {
-    const int at = o;
-    o += (n + 3) & ~3;
-    return at;
-  };
-  L.wt2 = take(d.C1 * SK * L.p2);
-  L.wt3 = take(d.C2 * SK * L.p3);
-  L.x = take(d.L0);
-  L.w1 = take(d.C1 * SK);
-  L.a1 = take(d.C1 * L.s1);
-  L.a2 = take(d.C2 * L.s2);
-  L.a3 = take(d.C3 * L.s3);
-  L.d2 = train ? take(d.C2 * L.s2) : o;
-  L.d1 = train ? take(d.C1 * L.s1) : o;
-  L.h0 = take(d.C3 + d.NS);
-  L.a4 = take(d.H);
-  L.a5 = take(d.H);
-  L.z = take(d.NOUT > d.H ? d.NOUT : d.H);
-  const int widest = d.H > d.C3 + d.NS ? d.H : d.C3 + d.NS;
-  L.g = train ? take(4 * ST > widest ? 4 * ST : widest) : o;
-  L.total = o;
-  return L;
-}
-
-constexpr int SAMPLE_SMEM = 200 * 1024;
-
-bool sample_fits(const Dims& d, bool train) {
-  return d.K == SK && d.S == SS && (size_t)sample_layout(d, train).total * sizeof(float) <= SAMPLE_SMEM;
-}
 
 // W (Cout, Cin, 5) -> wt[(c 5 + k) Cp + o], zero-padded to Cp channels (coalesced
 // reads, four in flight per thread; the scattered stores stay in shared memory)

@@ -1,0 +1,53 @@
+"""Workspace of the surrogate's calls: the convolutions' per-sample partial gradients
+are part of it only for networks that a kernel forms them for (kernel size 5, stride
+2, small enough for shared memory); every other network needs its activations alone.
+A workspace for a batch also serves every smaller one."""
+import ctypes as C
+
+import pytest
+
+from paper_1812_10375_gb300 import build
+
+
+@pytest.fixture(scope="module")
+def sur():
+    build.build()
+    from paper_1812_10375_gb300 import surrogate
+    return surrogate
+
+
+def al(n):
+    return (n + 63) & ~63
+
+
+def activations(L0, C1, C2, C3, K, S, NS, H, NOUT, B):
+    """Bytes of the layers' values and gradients and of the two loss terms."""
+    lens = []
+    for _ in range(3):
+        L0 = (L0 - K) // S + 1
+        lens.append(L0)
+    conv = [B * c * n for c, n in zip((C1, C2, C3), lens)]
+    h0, h, y = B * (C3 + NS), B * H, B * NOUT
+    return 4 * (3 * sum(map(al, conv)) + 2 * al(h0) + 6 * al(h) + 2 * al(y) + al(2))
+
+
+def workspace(sur, sizes, B):
+    return int(sur._lib().hlb_sur_workspace_bytes(C.byref(sur.hlb_sur_config(*sizes)), B))
+
+
+@pytest.mark.parametrize("sizes", [
+    (500, 16, 32, 32, 3, 2, 2, 256, 6), (500, 16, 32, 32, 5, 1, 2, 256, 6),  # another kernel size, another stride
+    (500, 16, 512, 512, 5, 2, 2, 256, 6), (4000, 16, 32, 32, 5, 2, 2, 256, 6)])  # too large for shared memory
+@pytest.mark.parametrize("B", [1, 256])
+def test_networks_by_layers_need_no_partials(sur, sizes, B):
+    assert workspace(sur, sizes, B) == activations(*sizes, B)
+
+
+def test_networks_by_samples_have_their_partials(sur):
+    sizes = (500, 16, 32, 32, 5, 2, 2, 256, 6)
+    conv = 16 * 5 + 16 + 32 * 16 * 5 + 32 + 32 * 32 * 5 + 32
+    last = 0
+    for B in range(1, 300):
+        n = workspace(sur, sizes, B)
+        assert n >= activations(*sizes, B) + 4 * B * conv and n >= last
+        last = n
