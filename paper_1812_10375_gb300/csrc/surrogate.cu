@@ -60,34 +60,37 @@ size_t al(size_t n) { return (n + 63) & ~(size_t)63; }  // 256-byte aligned floa
 // What the per-sample kernels (below) need of a network.
 constexpr int SK = 5, SS = 2, ST = 512;  // taps, stride, threads
 
+template <class I>
 struct SampleLayout {  // shared-memory offsets (floats); rows of odd length
-  int s1, s2, s3, p2, p3;
-  int x, w1, wt2, wt3, a1, a2, a3, d2, d1, h0, a4, a5, z, g, total;
+  I s1, s2, s3, p2, p3;
+  I x, w1, wt2, wt3, a1, a2, a3, d2, d1, h0, a4, a5, z, g, total;
 };
 
-__host__ __device__ inline SampleLayout sample_layout(const Dims& d, bool train) {
-  SampleLayout L;
+// I = int for networks that fit, whose sums do.
+template <class I>
+__host__ __device__ inline SampleLayout<I> sample_layout(const Dims& d, bool train) {
+  SampleLayout<I> L;
   L.s1 = d.L1 | 1;
   L.s2 = d.L2 | 1;
   L.s3 = d.L3 | 1;
   L.p2 = (d.C2 + 7) & ~7;
   L.p3 = (d.C3 + 7) & ~7;
-  int o = 0;
-  auto take = [&](int n) {
-    const int at = o;
+  I o = 0;
+  auto take = [&](I n) {
+    const I at = o;
     o += (n + 3) & ~3;
     return at;
   };
-  L.wt2 = take(d.C1 * SK * L.p2);
-  L.wt3 = take(d.C2 * SK * L.p3);
+  L.wt2 = take((I)d.C1 * SK * L.p2);
+  L.wt3 = take((I)d.C2 * SK * L.p3);
   L.x = take(d.L0);
-  L.w1 = take(d.C1 * SK);
+  L.w1 = take((I)d.C1 * SK);
   L.a1 = take(d.C1 * L.s1);
   L.a2 = take(d.C2 * L.s2);
   L.a3 = take(d.C3 * L.s3);
   L.d2 = train ? take(d.C2 * L.s2) : o;
   L.d1 = train ? take(d.C1 * L.s1) : o;
-  L.h0 = take(d.C3 + d.NS);
+  L.h0 = take((I)d.C3 + d.NS);
   L.a4 = take(d.H);
   L.a5 = take(d.H);
   L.z = take(d.NOUT > d.H ? d.NOUT : d.H);
@@ -100,7 +103,12 @@ __host__ __device__ inline SampleLayout sample_layout(const Dims& d, bool train)
 constexpr int SAMPLE_SMEM = 200 * 1024;
 
 bool sample_fits(const Dims& d, bool train) {
-  return d.K == SK && d.S == SS && (size_t)sample_layout(d, train).total * sizeof(float) <= SAMPLE_SMEM;
+  if (d.K != SK || d.S != SS) return false;
+  // every size is at least an array's; after that no product leaves 64 bits
+  constexpr int MOST = SAMPLE_SMEM / (int)sizeof(float);
+  for (const int n : {d.L0, d.C1, d.C2, d.C3, d.NS, d.H, d.NOUT})
+    if (n > MOST) return false;
+  return sample_layout<long long>(d, train).total <= MOST;
 }
 
 struct Acts {  // workspace offsets (floats)
@@ -586,7 +594,7 @@ __global__ void __launch_bounds__(ST, 1) k_sample(const Dims d, const Offsets o,
                                                   float* __restrict__ y, const float* __restrict__ target,
                                                   const int* __restrict__ label, const SampleOut out) {
   extern __shared__ __align__(16) float sm[];
-  const SampleLayout L = sample_layout(d, TRAIN);
+  const SampleLayout<int> L = sample_layout<int>(d, TRAIN);
   const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, W0 = d.C3 + d.NS;
   float *x = sm + L.x, *w1 = sm + L.w1, *wt2 = sm + L.wt2, *wt3 = sm + L.wt3, *a1 = sm + L.a1, *a2 = sm + L.a2,
         *a3 = sm + L.a3, *h0 = sm + L.h0, *a4 = sm + L.a4, *a5 = sm + L.a5, *z = sm + L.z;
@@ -771,7 +779,7 @@ int sample_grad_blocks(const Dims& d, const Offsets& o) {
 template <bool TRAIN>
 hlb_status launch_sample(const Dims& d, const Offsets& o, const float* P, const float* hist, const float* scal, int B,
                          float* y, const float* target, const int* label, const SampleOut& out, cudaStream_t s) {
-  const size_t smem = (size_t)sample_layout(d, TRAIN).total * sizeof(float);
+  const size_t smem = (size_t)sample_layout<int>(d, TRAIN).total * sizeof(float);
   if (cudaFuncSetAttribute(k_sample<TRAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, SAMPLE_SMEM) != cudaSuccess)
     return HLB_ECUDA;
   k_sample<TRAIN><<<B, ST, smem, s>>>(d, o, P, hist, scal, y, target, label, out);

@@ -43,6 +43,14 @@ def test_networks_by_layers_need_no_partials(sur, sizes, B):
     assert workspace(sur, sizes, B) == activations(*sizes, B)
 
 
+@pytest.mark.parametrize("sizes", [
+    (1636177817, 1, 1, 1, 5, 2, 1, 8, 2), (858993259, 2, 2, 8, 5, 2, 1, 8, 2), (572662106, 4, 4, 4, 5, 2, 1, 8, 2),
+    (409044304, 1, 1, 64, 5, 2, 1, 8, 2)])
+def test_layers_beyond_32_bits_do_not_fit_shared_memory(sur, sizes):
+    """Sizes of 2^32 floats and a few more: taken modulo 2^32 they are a few KB."""
+    assert workspace(sur, sizes, 1) == activations(*sizes, 1)
+
+
 def test_networks_by_samples_have_their_partials(sur):
     sizes = (500, 16, 32, 32, 5, 2, 2, 256, 6)
     conv = 16 * 5 + 16 + 32 * 16 * 5 + 32 + 32 * 32 * 5 + 32
