@@ -16,7 +16,10 @@
  *  - Pointers named d_* are CUDA device pointers; h_* are host pointers.
  *  - The caller owns every buffer and the stream.  The library never allocates
  *    device memory: it works inside the workspace the caller passes to
- *    hlb_init / hlb_batch_init, which must stay valid until hlb_destroy.
+ *    hlb_init / hlb_batch_init, which must stay valid until hlb_destroy.  On the
+ *    host it holds the handles, small tables, and one page-locked block of 64 KB
+ *    for the process (diagnostics records; from the first handle on, until the
+ *    process ends).
  *  - Host pointers are read or written only during the call.
  *  - Every call returns an hlb_status and never throws or aborts.  Kernels are
  *    launched asynchronously on the handle's stream; hlb_diag and the flux

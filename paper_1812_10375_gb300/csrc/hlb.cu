@@ -5,6 +5,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <mutex>
 #include <new>
 #include <vector>
 
@@ -433,7 +434,7 @@ struct hlb_domain {
   float* ftop[2] = {nullptr, nullptr};
   double* partials = nullptr;
   DevState* state = nullptr;
-  DevState* pin = nullptr;  // page-locked host copy of the record (hlb_diag)
+  DevState* pin = nullptr;  // page-locked host copy of the record (hlb_diag), or null
   double* hist = nullptr;
   // N > 1 (Eq. 27): rho^n, u_x^n, u_y^n of the step, a T buffer and the
   // sub-steps' per-block partials
@@ -676,25 +677,49 @@ hlb_status set_fields_at(hlb_domain* d, const float* d_rho, const float* d_T, in
   return HLB_OK;
 }
 
-// Page-locked host memory for n diagnostics records; null (hlb_diag then copies
-// through pageable memory) if there is none to be had.  Both calls run in the
-// relaxed capture mode: they touch no stream, and another thread's capture of its
-// own stream stays valid.
 struct RelaxedCapture {
   cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
   RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
   ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
 };
-DevState* pinned_records(int n) {
-  RelaxedCapture relaxed;
-  void* p = nullptr;
-  if (cudaHostAlloc(&p, (size_t)n * sizeof(DevState), cudaHostAllocDefault) == cudaSuccess) return (DevState*)p;
-  cudaGetLastError();
-  return nullptr;
+
+// Page-locked host records that hlb_diag copies into: one block of 64 KB for the
+// process, locked by the first handle and kept until the process ends, since
+// unlocking it would wait for all work on the device (a handle that owned its record
+// waited so in hlb_destroy, 118 ms behind another stream's work; giving the record back
+// takes 1 us).  A handle without a record (more than RECORDS domains at once, or no
+// memory to lock) reads through pageable memory.  The lock runs in the relaxed
+// capture mode: it touches no stream, and another thread's capture of its own
+// stream stays valid.
+constexpr int RECORDS = 512;
+struct RecordPool {
+  std::mutex mutex;
+  DevState* block;
+  DevState* free[RECORDS];
+  int n;
+};
+RecordPool g_records{};
+DevState* take_record() {
+  RecordPool& p = g_records;
+  std::lock_guard<std::mutex> lock(p.mutex);
+  if (!p.block) {
+    constexpr size_t PAGE = 1 << 16, BYTES = (RECORDS * sizeof(DevState) + PAGE - 1) / PAGE * PAGE;
+    void* const m = aligned_alloc(PAGE, BYTES);
+    RelaxedCapture relaxed;
+    if (!m || cudaHostRegister(m, BYTES, cudaHostRegisterPortable) != cudaSuccess) {
+      cudaGetLastError();
+      free(m);
+      return nullptr;
+    }
+    p.block = (DevState*)m;
+    for (; p.n < RECORDS; ++p.n) p.free[p.n] = p.block + p.n;
+  }
+  return p.n > 0 ? p.free[--p.n] : nullptr;
 }
-void free_records(DevState* p) {
-  RelaxedCapture relaxed;
-  if (p) cudaFreeHost(p);
+void give_record(DevState* r) {
+  if (!r) return;
+  std::lock_guard<std::mutex> lock(g_records.mutex);
+  g_records.free[g_records.n++] = r;
 }
 
 hlb_status init_domain(hlb_domain* d, const hlb_params* p, char* ws, cudaStream_t stream) {
@@ -1442,7 +1467,7 @@ hlb_status hlb_init(hlb_domain** out, const hlb_params* p, void* d_workspace, si
     delete d;
     return st;
   }
-  d->pin = pinned_records(1);
+  d->pin = take_record();
   *out = d;
   return HLB_OK;
 }
@@ -1566,7 +1591,7 @@ hlb_status hlb_reset_timeavg(hlb_domain* d) {
 hlb_status hlb_destroy(hlb_domain* d) {
   if (!d) return HLB_EINVAL;
   drop_graph(d);
-  free_records(d->pin);
+  give_record(d->pin);
   delete d;
   return HLB_OK;
 }
@@ -1656,8 +1681,7 @@ hlb_status hlb_batch_init(hlb_batch** out, int n, const hlb_params* p, void* d_w
     delete b;
     return st;
   }
-  DevState* const pin = pinned_records(n);
-  for (int i = 0; pin && i < n; ++i) b->dom[i].pin = pin + i;
+  for (auto& d : b->dom) d.pin = take_record();
   *out = b;
   return HLB_OK;
 }
@@ -1810,8 +1834,10 @@ hlb_status hlb_batch_checkpoint_load(hlb_batch* b, int i, const void* h_buf, siz
 hlb_status hlb_batch_destroy(hlb_batch* b) {
   if (!b) return HLB_EINVAL;
   batch_drop_graph(b);
-  for (auto& d : b->dom) drop_graph(&d);
-  free_records(b->dom[0].pin);
+  for (auto& d : b->dom) {
+    drop_graph(&d);
+    give_record(d.pin);
+  }
   delete b;
   return HLB_OK;
 }
