@@ -55,6 +55,8 @@ constexpr int NVARIANTS = (int)(sizeof(VARIANTS) / sizeof(VARIANTS[0]));
 constexpr int TILE_Y = 28;      // the default variant's tile height (variant 0)
 constexpr int MIN_TILE_Y = 16;  // the shortest variant tile (sizes the partial-sum slots)
 
+// The kernel of a chained step, with the reduction arguments of the step before.
+using ChainKernel = void (*)(StepArgs, SplitReduceArgs, int);
 // A compiled flow kernel: its tile's fluid rows and threads.
 struct FlowKernel {
   int ty, nth;
@@ -64,8 +66,7 @@ struct FlowKernel {
   void (*launch_single)(dim3, size_t, cudaStream_t, const StepArgs&);
   void (*launch_batch)(int, size_t, cudaStream_t, const StepArgs&, const DomArgs*, const int2*, const int*,
                        const float2*);
-  // a chained step, with the reduction arguments of the step before; may be null
-  void (*launch_chain)(dim3, size_t, cudaStream_t, const StepArgs&, const SplitReduceArgs&);
+  ChainKernel (*chain_kernel)(int nf);  // a chained step's kernel for nf partials; may be null
 };
 struct FlowVariant {
   int fk;      // flow kernel (index into FLOW_KERNELS), or -1: by flow_kernel_for()
@@ -93,17 +94,14 @@ void launch_flow_batch(int blocks, size_t smem, cudaStream_t s, const StepArgs& 
   k_flow_batch<TY, NTH, MINB, RP><<<blocks, NTH, smem, s>>>(phys, desc, blk, act, lag);
 }
 template <int TY, int NTH, int MINB, bool RP>
-void launch_flow_chain(dim3 grid, size_t smem, cudaStream_t s, const StepArgs& a, const SplitReduceArgs& r) {
-  grid.y += 1;
-  if (r.nf <= CHAIN_FEW)
-    k_flow_chain<TY, NTH, MINB, RP, CHAIN_FEW><<<grid, NTH, smem, s>>>(a, r, HIST_CAP);
-  else
-    k_flow_chain<TY, NTH, MINB, RP, CHAIN_PARTS><<<grid, NTH, smem, s>>>(a, r, HIST_CAP);
+ChainKernel chain_kernel_for(int nf) {
+  return nf <= CHAIN_FEW ? (ChainKernel)k_flow_chain<TY, NTH, MINB, RP, CHAIN_FEW>
+                         : (ChainKernel)k_flow_chain<TY, NTH, MINB, RP, CHAIN_PARTS>;
 }
 template <int TY, int NTH, int MINB, bool RP>
-constexpr auto flow_chain() -> decltype(FlowKernel::launch_chain) {
+constexpr auto flow_chain() -> decltype(FlowKernel::chain_kernel) {
   if constexpr (TY <= CHAIN_TY && RP)
-    return launch_flow_chain<TY, NTH, MINB, RP>;
+    return chain_kernel_for<TY, NTH, MINB, RP>;
   else
     return nullptr;
 }
@@ -551,7 +549,7 @@ SplitReduceArgs reduce_args_of(const hlb_domain* d, int part = 0) {
 
 // Whether the steps of one call are chained (hlb_split.cuh).
 bool chains(const hlb_domain* d) {
-  return flow_kernel_of(d).launch_chain && (long long)d->grid.x * d->grid.y <= CHAIN_PARTS;
+  return flow_kernel_of(d).chain_kernel && (long long)d->grid.x * d->grid.y <= CHAIN_PARTS;
 }
 
 // One step of the split form: the flow kernel, N energy sub-steps, the reduction.
@@ -565,9 +563,11 @@ hlb_status launch_split_step(hlb_domain* d, bool first, bool last, cudaEvent_t a
   const bool chain = chains(d);
   const int part = chain ? d->parity : 0;
   a.fpart = d->fpart[part];
-  if (chain && !first)
-    fl.launch_chain(d->grid, fl.smem, d->stream, a, reduce_args_of(d, part ^ 1));
-  else
+  if (chain && !first) {
+    // one row of blocks more than the tiles': its first updates the record
+    const SplitReduceArgs before = reduce_args_of(d, part ^ 1);
+    fl.chain_kernel(before.nf)<<<dim3(d->grid.x, d->grid.y + 1), fl.nth, fl.smem, d->stream>>>(a, before, HIST_CAP);
+  } else
     fl.launch_single(d->grid, fl.smem, d->stream, a);
   if (after_flow && cudaEventRecord(after_flow, d->stream) != cudaSuccess) return HLB_ECUDA;
   const int nsub = d->p.n_sub;
@@ -1862,9 +1862,16 @@ hlb_status hlb_autotune(hlb_domain* d, int steps_per_variant, int* chosen, float
     }
     set_variant_grids(d, v);
     drop_graph(d);
-    st = launch_step(d);  // one untimed step per variant (first-launch costs)
+    // one untimed step per variant (first-launch costs), then steps as hlb_step runs
+    // them: chained where the variant's are
+    st = launch_step(d);
+    if (st == HLB_OK && is_split(v) && chains(d)) {
+      cudaFuncAttributes loaded;  // (a single step does not launch, and so load, the chained kernel)
+      const ChainKernel k = flow_kernel_of(d).chain_kernel(reduce_args_of(d).nf);
+      if (cudaFuncGetAttributes(&loaded, (const void*)k) != cudaSuccess) st = HLB_ECUDA;
+    }
     cudaEventRecord(e0, d->stream);
-    for (int k = 0; k < steps_per_variant && st == HLB_OK; ++k) st = launch_step(d);
+    for (int k = 0; k < steps_per_variant && st == HLB_OK; ++k) st = launch_step(d, k == 0, k == steps_per_variant - 1);
     cudaEventRecord(e1, d->stream);
     float ms = 0.f;
     if (st == HLB_OK && (cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess))
