@@ -111,6 +111,35 @@ bool sample_fits(const Dims& d, bool train) {
   return sample_layout<long long>(d, train).total <= MOST;
 }
 
+// Whether a call runs by samples.  One CTA reads all linear weights for one sample and
+// stages all convolution weights: that pays while the linear layers are narrow and,
+// for many samples, the convolutions long.  Layers' time over samples' time on either
+// side of the lines (conv, lin: multiply-adds of a sample; channels 16/32/32 unless
+// short: conv = 4k):
+//  - training, lin: 1 sample, H = 1024 1.00, H = 1280 0.61; 256 samples, lin = 7 conv 1.39,
+//    15 conv 0.92.  4,096 samples, short: H = 512 1.00, H = 768 0.86.
+//  - training, rows of F2 that are not whole 16-byte pieces (read by 4 bytes): 153
+//    samples, H = 256 1.52, H = 512 0.74.
+//  - forward, lin: 1 sample, H = 1280 1.31 (short 1.23), H = 2048 0.97 (0.76); 64 samples,
+//    H = 2048 1.52 (1.28), 153 samples, short, H = 3072 0.99.
+//  - forward, conv: 1,024 samples, 106k 1.10, short 0.86; 4,096 samples, 306k 1.58,
+//    106k 0.83.
+//  - forward, NOUT = 1000 1.59, 8,000 0.59.
+constexpr int SAMPLE_BATCH = 512;
+bool by_samples(const Dims& d, int B, bool train) {
+  if (!sample_fits(d, train)) return false;
+  const long long conv = (long long)SK * (d.C1 * d.L1 + (long long)d.C1 * d.C2 * d.L2 + (long long)d.C2 * d.C3 * d.L3);
+  const long long lin = (long long)d.H * (d.C3 + d.NS + d.H + d.NOUT);
+  const bool whole = d.H % 4 == 0 && param_offsets(d).F2 % 4 == 0, many = B > SAMPLE_BATCH;
+  if (!train) {
+    if (d.NOUT > 1024 || (many && conv < 100000) || (B > 2 * SAMPLE_BATCH && conv < 300000)) return false;
+    return lin <= 1700000 || (B >= 64 && lin <= 5000000 && whole);
+  }
+  if (!whole) return lin <= 80000 && !(many && conv < 100000);
+  if (many && conv < 100000) return lin <= 300000;
+  return lin <= 1100000 || (B >= 256 && lin <= 8 * conv);
+}
+
 struct Acts {  // workspace offsets (floats)
   size_t z1, a1, z2, a2, z3, a3, h0, z4, a4, z5, a5, y, dy, dz5, dz4, dh0, dz3, dz2, dz1, loss, part, total;
 };
@@ -139,10 +168,13 @@ Acts act_offsets(const Dims& d, int B) {
   a.dz3 = p; p += al(n3);
   a.dz2 = p; p += al(n2);
   a.dz1 = p; p += al(n1);
-  // by samples: a pair of loss terms and the convolutions' partial gradients of each
-  const bool samples = sample_fits(d, true);
-  a.loss = p; p += al(samples ? 2 * (size_t)B : 2);
-  a.part = p; p += samples ? al((size_t)B * param_offsets(d).F1) : 0;
+  // by samples: a pair of loss terms and the convolutions' partial gradients of each.  (A
+  // workspace for B serves every smaller batch; one beyond SAMPLE_BATCH may run by
+  // layers where those up to it run by samples.)
+  const int most = by_samples(d, B, true) ? B : B < SAMPLE_BATCH ? B : SAMPLE_BATCH;
+  const bool samples = by_samples(d, most, true);
+  a.loss = p; p += al(samples ? 2 * (size_t)most : 2);
+  a.part = p; p += samples ? al((size_t)most * param_offsets(d).F1) : 0;
   a.total = p;
   return a;
 }
@@ -373,8 +405,8 @@ __global__ void k_adam(long long n, float* __restrict__ p, const float* __restri
 // ------------------------------------------------- one CTA per sample
 // Forward pass, loss and data gradients of one sample in one CTA, with every
 // activation in shared memory, for the framework's kernel size and stride (K = 5,
-// S = 2) and networks that fit.  The layer-by-layer kernels above take any other
-// sizes; on a batch of 64 their 21 launches cost more than their arithmetic (243
+// S = 2) and networks that fit and are narrow enough (by_samples).  The layer-by-layer
+// kernels above take any other sizes; on a batch of 64 their 21 launches cost more than their arithmetic (243
 // MFLOP), and the convolutions' inner loops read every operand from L1.  Here a
 // thread forms eight output channels of one position from one input value and two
 // broadcast 16-byte weight loads per tap, so that the FP32 pipe and shared memory
@@ -877,7 +909,7 @@ hlb_status hlb_sur_forward(const hlb_sur_config* c, const float* d_params, const
   const Acts A = act_offsets(d, B);
   float* w = (float*)d_ws;
   cudaStream_t s = (cudaStream_t)stream;
-  if (sample_fits(d, false)) {
+  if (by_samples(d, B, false)) {
     const hlb_status st = launch_sample<false>(d, o, d_params, d_hist, d_scal, B, d_out, nullptr, nullptr, SampleOut{}, s);
     if (st != HLB_OK) return st;
     return cudaGetLastError() == cudaSuccess ? HLB_OK : HLB_ECUDA;
@@ -902,7 +934,7 @@ hlb_status hlb_sur_loss_grad(const hlb_sur_config* c, const float* d_params, con
   const float* P = d_params;
   float* G = d_grad;
   cudaStream_t s = (cudaStream_t)stream;
-  if (sample_fits(d, true)) {
+  if (by_samples(d, B, true)) {
     const SampleOut out = {w + A.h0, w + A.a4, w + A.dz4, w + A.a5, w + A.dz5, w + A.dy, w + A.part, w + A.loss};
     const hlb_status st = launch_sample<true>(d, o, P, d_hist, d_scal, B, nullptr, d_target, d_label, out, s);
     if (st != HLB_OK) return st;

@@ -59,3 +59,35 @@ def test_networks_by_samples_have_their_partials(sur):
         n = workspace(sur, sizes, B)
         assert n >= activations(*sizes, B) + 4 * B * conv and n >= last
         last = n
+
+
+def with_partials(sizes, B, samples):
+    """Workspace bytes for a batch of B with partial gradients of `samples` samples."""
+    L0, C1, C2, C3, K, S, NS, H, NOUT = sizes
+    conv = C1 * K + C1 + C2 * C1 * K + C2 + C3 * C2 * K + C3
+    return activations(*sizes, B) + (4 * (al(2 * samples) - al(2) + al(samples * conv)) if samples else 0)
+
+
+@pytest.mark.parametrize("sizes,batches", [
+    # wide linear layers: by layers, but for large batches behind long convolutions
+    ((500, 16, 32, 32, 5, 2, 3, 1024, 6), {1: 1, 256: 256, 4096: 4096}),
+    ((500, 16, 32, 32, 5, 2, 3, 1280, 6), {1: 0, 255: 0, 256: 256, 4096: 4096}),
+    ((500, 16, 32, 32, 5, 2, 3, 2048, 6), {1: 0, 255: 0, 256: 256, 4096: 4096}),
+    ((500, 16, 32, 32, 5, 2, 3, 3072, 6), {1: 0, 256: 0, 4096: 0}),
+    ((100, 16, 32, 32, 5, 2, 3, 1280, 6), {1: 0, 256: 0, 4096: 0}),
+    # short convolutions, not so narrow: by layers from 513 samples on, whose workspace serves 512
+    ((64, 4, 8, 8, 5, 2, 3, 768, 6), {512: 512, 513: 512, 4096: 512}),
+    ((64, 4, 8, 8, 5, 2, 3, 256, 6), {512: 512, 513: 513, 4096: 4096}),
+    ((100, 16, 32, 32, 5, 2, 3, 256, 6), {512: 512, 513: 513, 4096: 4096}),
+    # rows that are not whole 16-byte pieces: narrow layers only
+    ((500, 16, 32, 32, 5, 2, 3, 255, 6), {1: 1, 256: 256}), ((500, 16, 32, 32, 5, 2, 3, 510, 6), {1: 0, 256: 0}),
+    ((500, 16, 32, 33, 5, 2, 3, 512, 6), {1: 0, 256: 0}), ((500, 16, 32, 32, 5, 2, 3, 512, 6), {1: 1, 256: 256})])
+def test_which_batches_run_by_samples(sur, sizes, batches):
+    for B, samples in batches.items():
+        assert workspace(sur, sizes, B) == with_partials(sizes, B, samples), B
+
+
+def test_workspace_grows_with_the_batch(sur):
+    for sizes in [(64, 4, 8, 8, 5, 2, 3, 768, 6), (29, 1, 1, 1, 5, 2, 1, 8, 2), (500, 16, 32, 32, 5, 2, 3, 2048, 6)]:
+        n = [workspace(sur, sizes, B) for B in range(1, 4097)]
+        assert n == sorted(n)
