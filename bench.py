@@ -44,6 +44,7 @@ FLOW_BYTES_FLUID = 36 + 36 + 4 + 12
 ENERGY_BYTES_FLUID = 4 + 12 + 4
 ENERGY_BYTES_SOLID = 8
 KIND_SPLIT, KIND_FUSED, KIND_MARCH = 0, 1, 2
+ROWS_BY_SIZE = -2  # segment height of the one-warp walk: decided by the lattices
 
 KERNEL_SOURCES = ("hlb_internal.cuh", "hlb_kernels.cuh", "hlb_march.cuh", "hlb_split.cuh", "hlb_energy_walk.cuh",
                   "hlb_pair.cuh", "hlb_energy_pair.cuh")  # step kernels' device code
@@ -59,8 +60,10 @@ def kernel_source_hash() -> str:
 
 
 def energy_kernel_name(erows):
-    """The split step's energy kernel: the row-walking one (segments of erows
-    rows) or the tiled one (erows = 0)."""
+    """The split step's energy kernel: the one-warp walk (segments sized by the
+    lattices), the two-warp walk (segments of erows rows) or the tiled one (erows = 0)."""
+    if erows == ROWS_BY_SIZE:
+        return "k_energy_pair_batch"
     return "k_energy_walk_batch" if erows > 0 else "k_energy_batch"
 
 
@@ -74,10 +77,10 @@ def kernel_name(tile, kind=KIND_FUSED, erows=-1):
 
 def variant_key(tile, kind=KIND_FUSED, erows=-1):
     """Suffix naming a variant in the committed ncu summary: the tile, and for a
-    split variant its energy kernel (walk<rows> or tile)."""
+    split variant its energy kernel (pair, walk<rows> or tile)."""
     key = "x".join(str(t) for t in tile)
     if kind == KIND_SPLIT:
-        key += "_walk%d" % erows if erows > 0 else "_tile"
+        key += "_pair" if erows == ROWS_BY_SIZE else "_walk%d" % erows if erows > 0 else "_tile"
     return key
 
 
@@ -391,10 +394,7 @@ def run_ours(args):
     ms_per_step, value = aggregate(elapsed_ms, cells, args.steps, dist)
     kern_avg_ms = sum(kern_ms) / len(kern_ms)
     kernels = None
-    # variant 0 walks its rows by one warp, the other split variants by two
     step_names = kernel_name(variants[chosen], kind, erows).split("+")
-    if chosen == 0:
-        step_names[-1] = "k_energy_pair_batch"
     if kind == KIND_SPLIT:
         flow_ms = sum(ev_b[k].elapsed_time(ev_f[k]) for k in range(n_ev)) / n_ev
         en_ms = sum(ev_f[k].elapsed_time(ev_a[k]) for k in range(n_ev)) / n_ev
@@ -433,7 +433,7 @@ def run_ours(args):
                        "timing": "CUDA events on the batch stream around K graph-replayed steps; the step "
                                  "kernel bracketed per step over %d further launches for the roofline" % n_ev,
                        "tile": {"chosen": list(variants[chosen]), "chosen_index": chosen,
-                                "chosen_energy_walk_rows": erows,
+                                "chosen_energy_walk_rows": "by size" if erows == ROWS_BY_SIZE else erows,
                                 "candidates_w_h_threads": [list(v) for v in variants],
                                 "tuning_ms_per_step": [round(m, 4) for m in tune_ms]}},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",

@@ -328,7 +328,7 @@ hlb_status hlb_batch_destroy(hlb_batch* b);
  *    heights, then N energy sub-step kernels over strips of 56 columns: a walk
  *    up the rows by one warp (variant 0, the default for the finite-volume
  *    scheme: its segments and its flow tile are sized by the lattices, and the
- *    heights it reports are those of large ones) or by two warps (segments of 96
+ *    tile it reports is that of large ones) or by two warps (segments of 96
  *    or 64 rows), or a tiled kernel over 56 x 24 tiles;
  *  - HLB_KIND_FUSED: one fused step kernel over 52-column tiles of a few
  *    heights, with 256 or 512 threads per CTA (the default for the isotropic
@@ -341,17 +341,19 @@ hlb_status hlb_batch_destroy(hlb_batch* b);
  * a fused tiled one its tile's, a row-marching one width 0, its segment height
  * and 0 threads.  hlb_variant_kind(v) returns the kind of variant v, or -1;
  * hlb_variant_energy_rows(v) the segment height of a split variant's
- * row-walking energy kernel, 0 for a split variant with the tiled energy
- * kernel, -1 for the other kinds or v out of range.  hlb_autotune / hlb_batch_autotune run one untimed and
- * then steps_per_variant timed steps of every variant available to the
- * handle on its own state (others report 1e30 ms), keep the fastest for later
- * steps and report its index in *chosen (and the measured ms per step in
- * h_ms[0..max_out) if h_ms is not NULL).  The timed steps are ordinary steps of
+ * row-walking energy kernel, HLB_ROWS_BY_SIZE where the lattices' sizes decide it
+ * (variant 0: 4 to 256 rows), 0 for a split variant with the tiled energy kernel,
+ * -1 for the other kinds or v out of range.  hlb_autotune / hlb_batch_autotune
+ * run one untimed and then steps_per_variant timed steps of every variant
+ * available to the handle on its own state (others report 1e30 ms), keep the
+ * fastest for later steps and report its index in *chosen (and the measured ms
+ * per step in h_ms[0..max_out) if h_ms is not NULL).  The timed steps are ordinary steps of
  * the simulation: every variant evaluates a cell's update with the same
  * arithmetic (tiled shapes differ only in the order of the FP64 partial sums,
  * hence in the last bits of the mean density of Eq. 9; the two forms agree to
  * FP32 rounding).  Synchronises the stream. */
 enum { HLB_KIND_SPLIT = 0, HLB_KIND_FUSED = 1, HLB_KIND_MARCH = 2 };
+enum { HLB_ROWS_BY_SIZE = -2 };
 int hlb_tile_variants(int* h_tile_w, int* h_tile_h, int* h_threads, int max_out);
 int hlb_variant_kind(int v);
 int hlb_variant_energy_rows(int v);

@@ -1974,7 +1974,7 @@ int hlb_variant_kind(int v) {
 
 int hlb_variant_energy_rows(int v) {
   if (v < 0 || v >= NV_ALL || !is_split(v)) return -1;
-  return FLOWS[v].ewalk == 2 ? 64 : (FLOWS[v].ewalk ? FLOWS[v].ep : 0);
+  return FLOWS[v].ewalk == 2 ? HLB_ROWS_BY_SIZE : (FLOWS[v].ewalk ? FLOWS[v].ep : 0);
 }
 
 const char* hlb_strerror(hlb_status s) {

@@ -20,6 +20,7 @@ HLB_STORE_DEVIATION, HLB_STORE_PLAIN = 0, 1
 HLB_DIFF_FV, HLB_DIFF_ISO = 0, 1
 HLB_BOTTOM_DIRICHLET, HLB_BOTTOM_FLUX = 0, 1
 HLB_KIND_SPLIT, HLB_KIND_FUSED, HLB_KIND_MARCH = 0, 1, 2
+HLB_ROWS_BY_SIZE = -2
 TOP_KIND = {"wall": HLB_TOP_WALL, "const_rho": HLB_TOP_CONST_RHO, "convective": HLB_TOP_CONVECTIVE}
 
 
@@ -211,7 +212,8 @@ def variant_kinds():
 
 def variant_energy_rows():
     """Per compiled variant: the segment height of a split variant's row-walking
-    energy kernel, 0 for the tiled energy kernel, -1 for the fused kinds."""
+    energy kernel (HLB_ROWS_BY_SIZE where the lattices decide it), 0 for the tiled
+    energy kernel, -1 for the fused kinds."""
     n = lib().hlb_tile_variants(None, None, None, 0)
     return [int(lib().hlb_variant_energy_rows(k)) for k in range(n)]
 
