@@ -93,10 +93,13 @@ void launch_flow_batch(int blocks, size_t smem, cudaStream_t s, const StepArgs& 
                        const int2* blk, const int* act, const float2* lag) {
   k_flow_batch<TY, NTH, MINB, RP><<<blocks, NTH, smem, s>>>(phys, desc, blk, act, lag);
 }
+// 8-row tiles are taken where 4-row ones are more than are resident at once, so they
+// are never few.
 template <int TY, int NTH, int MINB, bool RP>
 ChainKernel chain_kernel_for(int nf) {
-  return nf <= CHAIN_FEW ? (ChainKernel)k_flow_chain<TY, NTH, MINB, RP, CHAIN_FEW>
-                         : (ChainKernel)k_flow_chain<TY, NTH, MINB, RP, CHAIN_PARTS>;
+  if constexpr (TY != 8)
+    if (nf <= CHAIN_FEW) return k_flow_chain<TY, NTH, MINB, RP, CHAIN_FEW>;
+  return k_flow_chain<TY, NTH, MINB, RP, CHAIN_PARTS>;
 }
 template <int TY, int NTH, int MINB, bool RP>
 constexpr auto flow_chain() -> decltype(FlowKernel::chain_kernel) {
