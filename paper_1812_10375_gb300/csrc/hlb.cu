@@ -212,9 +212,9 @@ static_assert(EW_OUT == EN_TX && EP_OUT == EN_TX, "walk strips and energy tiles 
 // once.  A warp's rows follow one another (about 0.3 us a row alone, 0.6 us with two
 // warps on a scheduler), so short segments win until the chip is full; beyond that a
 // second wave costs more than taller segments.  The energy kernel on the 32-domain
-// sweep, by segments (an earlier form of it, 10% faster throughout): 1,142 of 86 rows
-// 0.059 ms, 901 of 112 0.070, 1,815 of 54 0.072; on 14 lattices of 400 x 600: 1,120 of
-// 60 rows 0.047 ms, 1,792 of 38 0.055.
+// sweep, by segments: 1,142 of 86 rows 0.066 ms, 901 of 112 0.078, 1,815 of 54 0.082; on
+// 14 lattices of 400 x 600: 1,120 of 60 rows 0.052 ms, 896 of 76 0.058, 1,792 of 38
+// 0.064.
 int walk_rows(int n, const int* strips, const int* ny) {
   auto segments = [&](int L) {
     long long w = 0;

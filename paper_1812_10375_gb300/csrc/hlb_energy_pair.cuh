@@ -12,9 +12,11 @@
 // the row y + 1 value was produced earlier in the same walk step.
 //
 // The arithmetic of a cell is that of the tiled and the two-warp kernels
-// (hlb_split.cuh, hlb_energy_walk.cuh), operation by operation and rounding by
-// rounding: both columns of a packed instruction round on their own, so the new
-// temperature is the same bit for bit.
+// (hlb_split.cuh, hlb_energy_walk.cuh), operation by operation and, for a lattice by
+// itself, rounding by rounding: both columns of a packed instruction round on their
+// own, so its new temperature is the same bit for bit.  A batch sums two
+// conductivities with one rounding less in half of its rows (pair_step), so its
+// cells agree with a lattice by itself to FP32 rounding only.
 //
 // Why this shape: the update is bound by instruction issue and by the latency of a
 // row's dependent stages, not by memory (20 B per cell).  Two columns per lane make
@@ -223,8 +225,12 @@ __device__ __forceinline__ void pair_step(const StepArgs& A, const PairCtx& C, P
     if constexpr (BATCH) {
       // Sums of the row's lambda with a neighbour's: rows 4k and 4k + 1 add the
       // product rho (cv k) unrounded (one multiply-add), the others its rounded
-      // value.  The two-warp walk rounded so (in its groups of four interior rows,
-      // 64 rows to a segment); a batch's fields stay the same bit for bit.
+      // value.  The two-warp walk's batch form rounds so (as the compiler contracted
+      // its groups of four interior rows, 64 rows to a segment), and a batch here
+      // follows it but for single roundings next to those segments' edges: 1 of 4.9 M
+      // temperatures of the 32-domain sweep after three steps, 4e-7 of the largest
+      // value after 100.  It costs five reciprocals a row, which the other form shares
+      // between the columns and rows.
       const int tq = y & ~3;
       const bool fused = !(y & 2) && (tq & 63) && tq >= W + 7 && tq <= ny - 7;
       const float2 sa = fused ? rho1 : l;

@@ -1,7 +1,7 @@
 // Two neighbouring columns per thread: packed FP32 arithmetic (one instruction
 // for both columns on sm_100 and later) and the exchange of edge columns inside
-// a warp.  Every operation is written out (no compiler contraction), so that a
-// cell's update rounds the same way in every kernel form that contains it.
+// a warp.  Every operation is written out (no compiler contraction), so that where a
+// cell's update rounds is decided by its source, not by the loop it stands in.
 #pragma once
 #include "hlb_internal.cuh"
 
